@@ -249,9 +249,10 @@ int finish_on_single_path(pdhgc_batch* B, int k, int mode, const pdhgc_params& p
   BCK(cudaStreamCreateWithFlags(&st, cudaStreamNonBlocking));
   const auto& h = B->host[k];
   pdhgc_lp* lp = nullptr;
-  int rc = pdhgc_lp_create(&lp, h.m, h.n, (int64_t)h.col.size(), h.rp.data(), h.col.data(), h.val.data(),
+  int rc = lp_create(&lp, h.m, h.n, (int64_t)h.col.size(), h.rp.data(), h.col.data(), h.val.data(),
                            h.b.data(), h.c.data(), h.lb.empty() ? nullptr : h.lb.data(),
-                           h.ub.empty() ? nullptr : h.ub.data(), h.sense.empty() ? nullptr : h.sense.data(), 0, st);
+                           h.ub.empty() ? nullptr : h.ub.data(), h.sense.empty() ? nullptr : h.sense.data(), 0, st,
+                     false);
   pdhgc_report r1{}, rc_rep{};
   std::vector<double> x1(h.n), y1(h.m), xc(h.n), yc(h.m);
   if (rc == PDHGC_OK) rc = pdhgc_solve(lp, &p, &r1);

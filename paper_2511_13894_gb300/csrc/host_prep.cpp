@@ -2,7 +2,9 @@
 #include "host_prep.h"
 
 #include <algorithm>
+#include <climits>
 #include <cmath>
+#include <functional>
 #include <numeric>
 #include <thread>
 
@@ -203,6 +205,130 @@ void plan_chunks(const Csr& T, int32_t chunk, int32_t sms, ChunkPlan& P) {
     }
     ++waves;
   }
+}
+
+void plan_steps(const Csr& csr, int32_t ctas, bool bulk, StepPlan& P) {
+  P = StepPlan();
+  P.ctas = ctas;
+  auto len = [&](int32_t r) { return csr.row_ptr[r + 1] - csr.row_ptr[r]; };
+  while (P.hot < csr.rows && P.hot < kStepMaxHot && len(P.hot) >= kStepHotLen) ++P.hot;
+  struct Unit {
+    int32_t row, nrows, lg;
+    int64_t steps, parts;
+    int64_t cost;  // FP64 warp operations: steps, joining of lanes and parts, epilogue
+  };
+  std::vector<Unit> units;
+  auto add = [&](int32_t row, int32_t nrows, int32_t lg, int64_t steps, int64_t parts) {
+    const int64_t join = bulk && lg < 5 ? (1 << lg) - 1 : lg;
+    units.push_back({row, nrows, lg, steps, parts, parts * (steps + join + (parts > 1 ? 1 : 0)) + 5});
+  };
+  if (bulk) {
+    for (int32_t r = 0; r < csr.long_rows; ++r) {
+      const int32_t parts = r < csr.cta_rows ? kWarpsPerBlock : 1;
+      add(r, 1, 5, (len(r) + 32 * parts - 1) / (32 * parts), parts);
+    }
+    for (int32_t s = 0; s < csr.nslices; ++s) {
+      const int32_t w = csr.slice_w[s];
+      int32_t lg = 0;
+      while ((1 << lg) < kWarpsPerBlock && (kColsPerWarp << lg) < w) ++lg;
+      for (int32_t g = 0; g < (1 << lg); ++g) {
+        const int32_t row = csr.long_rows + s * kSellH + g * (kSellH >> lg);
+        if (row < csr.rows) add(row, std::min(kSellH >> lg, csr.rows - row), lg, (w + (1 << lg) - 1) >> lg, 1);
+      }
+    }
+  } else {
+    const int64_t warps = (int64_t)ctas * kStepWarps;
+    const int64_t cw = std::min<int64_t>(
+        std::max<int64_t>(((csr.nnz / 32 + warps - 1) / warps + 1) & ~int64_t(1), kStepMinCols), kStepMaxCols);
+    const int64_t ucap = std::max<int64_t>(cw, csr.nnz / 32 / ctas / 2);
+    for (int32_t r = 0; r < csr.rows;) {
+      int32_t lg = 0;
+      while (lg < 5 && ((len(r) + (1 << lg) - 1) >> lg) > ucap) ++lg;
+      const int32_t nr = std::min(32 >> lg, csr.rows - r);
+      const int64_t steps = (len(r) + (1 << lg) - 1) >> lg, parts = std::max<int64_t>(1, (steps + cw - 1) / cw);
+      const int64_t width = ((steps + parts - 1) / parts + 1) & ~int64_t(1);  // even: a part is whole pairs
+      add(r, nr, lg, width, std::max<int64_t>(1, (steps + width - 1) / std::max<int64_t>(width, 1)));
+      r += nr;
+    }
+  }
+  std::vector<int32_t> order(units.size());
+  std::iota(order.begin(), order.end(), 0);
+  std::stable_sort(order.begin(), order.end(), [&](int32_t a, int32_t b) { return units[a].cost > units[b].cost; });
+  using Load = std::pair<int64_t, int32_t>;
+  auto deal = [](std::vector<Load>& heap, int64_t cost) {  // to the least loaded
+    std::pop_heap(heap.begin(), heap.end(), std::greater<Load>());
+    const int32_t who = heap.back().second;
+    heap.back().first += cost;
+    std::push_heap(heap.begin(), heap.end(), std::greater<Load>());
+    return who;
+  };
+  std::vector<Load> heap;
+  for (int32_t b = 0; b < ctas; ++b) heap.push_back({0, b});
+  std::vector<std::vector<int32_t>> own(ctas);
+  for (int32_t u : order) own[deal(heap, units[u].cost)].push_back(u);
+  P.warp_ptr.push_back(0);
+  P.epi_ptr.push_back(0);
+  P.slot_ptr.push_back(0);
+  struct Task {
+    StepTask t;
+    StepSrcMap m;
+    int64_t cost;
+  };
+  std::vector<Task> all;
+  std::vector<Task> mine[kStepWarps];
+  for (int32_t b = 0; b < ctas; ++b) {
+    all.clear();
+    int64_t part = 0;
+    for (int32_t u : own[b]) {
+      const Unit& U = units[u];
+      if (U.steps > 2 * INT16_MAX || part + U.parts * U.nrows > INT32_MAX / 16) return;  // P.ok stays false
+      for (int64_t k = 0; k < U.parts; ++k) {
+        Task q{};
+        q.t.row = U.row;
+        q.t.slot = (int32_t)(part + k * U.nrows);
+        q.t.np = (int16_t)((U.steps + 1) / 2);
+        q.t.nrows = (uint8_t)U.nrows;
+        q.t.flags = (uint8_t)(U.lg | (U.parts > 1 ? kStepSplit : 0));
+        if (!bulk)
+          q.m = {1 << U.lg, 1, (int32_t)((k * U.steps) << U.lg), INT32_MAX};
+        else if (U.lg == 5)
+          q.m = {(int32_t)(32 * U.parts), 1, (int32_t)(32 * k), INT32_MAX};
+        else
+          q.m = {1, (int32_t)U.steps, 0, (int32_t)U.steps};
+        q.cost = U.steps + U.lg + (U.parts > 1 ? 1 : 5);
+        all.push_back(q);
+      }
+      if (U.parts > 1) {
+        P.epis.push_back(StepEpi{U.row, (int32_t)part, (int32_t)U.parts, (uint8_t)U.nrows, (uint8_t)U.lg, 0});
+        part += U.parts * U.nrows;
+      }
+    }
+    std::stable_sort(all.begin(), all.end(), [](const Task& x, const Task& y) { return x.cost > y.cost; });
+    heap.clear();
+    for (int32_t w = 0; w < kStepWarps; ++w) heap.push_back({0, w});
+    for (auto& v : mine) v.clear();
+    for (const Task& q : all) mine[deal(heap, q.cost)].push_back(q);
+    int64_t slots = 0;
+    for (auto& v : mine) {
+      for (Task& q : v) {
+        q.t.base = (int32_t)slots;
+        slots += (int64_t)q.t.np * 64;
+        if (P.nslots + slots > INT32_MAX - 64) return;
+        P.tasks.push_back(q.t);
+        P.map.push_back(q.m);
+        P.slot0.push_back((int32_t)P.nslots);
+      }
+      P.warp_ptr.push_back((int32_t)P.tasks.size());
+    }
+    P.nslots += slots;
+    P.max_tasks = std::max<int32_t>(P.max_tasks, (int32_t)all.size());
+    P.max_epis = std::max<int32_t>(P.max_epis, (int32_t)P.epis.size() - P.epi_ptr.back());
+    P.max_part = std::max<int32_t>(P.max_part, (int32_t)part);
+    P.max_slots = std::max<int32_t>(P.max_slots, (int32_t)slots);
+    P.epi_ptr.push_back((int32_t)P.epis.size());
+    P.slot_ptr.push_back((int32_t)P.nslots);
+  }
+  P.ok = true;
 }
 
 void plan_segments(Csr& csr) {

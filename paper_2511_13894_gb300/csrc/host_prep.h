@@ -104,6 +104,68 @@ struct ChunkPlan {
 // chunks of `chunk` (<= 65535) gathered entries on a GPU with `sms` SMs.
 void plan_chunks(const struct Csr& T, int32_t chunk, int32_t sms, ChunkPlan& out);
 
+// The persistent step kernel (steps.cuh): the work of a pass as tasks of one
+// warp, dealt to the CTAs longest first (each to the least loaded CTA) and by
+// each CTA to its warps in the same way.  A task sums R = 32 / L rows with L
+// lanes each (lane q * R + r: part q of row r); its steps are entries per lane.
+// Two plans:
+//   bulk (FP32 bulk): each row in exactly the order of the per-pass kernel.
+//     FP32 results are compared in all their bits, and every row sum is rounded
+//     to 48 bits.  A SELL slice of K parts (plan_segments) becomes K tasks of
+//     32 / K rows with a lane per row and part, added in part order; a warp row
+//     one task; a CTA row kWarpsPerBlock tasks of one CTA, joined in shared
+//     memory.  A step costs about a dozen FP32 instructions, so that up to 128
+//     steps in one warp are no bottleneck.
+//   fine (FP64): an FP64 operation takes its scheduler 64 cycles whatever its
+//     active lanes, so that the longest chain of steps is what counts: 200 x 500
+//     random-face LP 6.2 us per iteration in the bulk plan and 3.5 in this one,
+//     20k x 80k power law 19.7 and 13.5.  L is the smallest for which a unit is
+//     at most half a CTA's mean share of steps; one of more than the mean per
+//     warp (at least kStepMinCols) is cut into column parts of equal width,
+//     which meet in shared memory.  One lane per row costs the FP64 units least
+//     (no lane reduction, a full warp in the epilogue).
+constexpr int kStepThreads = 512;  // 128 registers a thread: with 1024 and 64 the FP64 operators spill
+constexpr int kStepWarps = kStepThreads / 32;
+constexpr int kStepMinCols = 4;
+constexpr int kStepMaxCols = 64;
+constexpr int kStepHotLen = 128;  // rows at least this long are hot: most SMs read their entry
+constexpr int kStepMaxHot = 4096;
+constexpr uint8_t kStepLgMask = 7;  // log2 of L
+constexpr uint8_t kStepSplit = 8;   // one of several tasks of its rows: their StepEpi runs the epilogue
+struct StepTask {
+  int32_t base;  // first slot, relative to the CTA's first slot (multiple of 64)
+  int32_t row;   // first row
+  int32_t slot;  // first partial sum, one per row (split)
+  int16_t np;    // pairs of steps
+  uint8_t nrows;
+  uint8_t flags;
+};
+struct StepEpi {
+  int32_t row;
+  int32_t slot;  // part k's row r at slot + k * nrows + r
+  int32_t k;     // parts
+  uint8_t nrows;
+  uint8_t lg;
+  int16_t pad;
+};
+struct StepSrcMap {  // entry of lane (q, r) in step j < jmax: j * sj + q * sq + off of row r
+  int32_t sj, sq, off, jmax;
+};
+struct StepPlan {
+  bool ok = false;  // false: beyond the kernel's index limits
+  int32_t ctas = 0;
+  int32_t hot = 0;  // leading rows of at least kStepHotLen entries (up to kStepMaxHot)
+  int32_t max_tasks = 0, max_epis = 0, max_part = 0, max_slots = 0;  // per CTA
+  int64_t nslots = 0;
+  std::vector<StepTask> tasks;
+  std::vector<StepEpi> epis;
+  std::vector<StepSrcMap> map;      // per task
+  std::vector<int32_t> slot0;       // per task: the CTA's first slot
+  std::vector<int32_t> warp_ptr;    // ctas * kStepWarps + 1: tasks of each warp
+  std::vector<int32_t> epi_ptr, slot_ptr;  // ctas + 1
+};
+void plan_steps(const struct Csr& csr, int32_t ctas, bool bulk, StepPlan& out);
+
 struct Prepared {
   int32_t m = 0, n = 0;
   int64_t nnz = 0;

@@ -101,6 +101,12 @@ struct SumD {
     for (int i = 0; i < NV; ++i) r.v[i] = __shfl_xor_sync(mask, v[i], off);
     return r;
   }
+  __device__ __forceinline__ SumD shfl_down(unsigned mask, int off) const {
+    SumD r;
+#pragma unroll
+    for (int i = 0; i < NV; ++i) r.v[i] = __shfl_down_sync(mask, v[i], off);
+    return r;
+  }
 };
 
 struct MaxD {
@@ -502,7 +508,8 @@ __device__ __forceinline__ void row_dot_global(const Op& op, typename Op::Acc& a
 }
 
 // Operators whose epilogue reads per-row inputs can declare `Pre`,
-// `prefetch(row)` and `epilogue_pre(row, acc, pre, part)`: the kernel then
+// `prefetch(row)` and `epilogue_pre(row, acc, pre, part)` (which returns the
+// row's entry of the vector that the other pass gathers): the kernel then
 // loads those inputs right after the grid-dependency wait, so that their
 // latency overlaps the gathers instead of following them.
 template <class Op, class = void>
@@ -524,11 +531,19 @@ struct Prefetcher<Op, std::void_t<typename Op::Pre>> {
   __device__ static void epilogue(const Op& op, int r, const typename Op::Acc& a, const Pre& p, double* part) {
     op.epilogue_pre(r, a, p, part);
   }
+  __device__ static typename Op::GT epilogue_val(const Op& op, int r, const typename Op::Acc& a, const Pre& p,
+                                                 double* part) {
+    return op.epilogue_pre(r, a, p, part);
+  }
 #else  // the same inputs, loaded when the epilogue runs
   struct Pre {};
   __device__ static Pre get(const Op&, int) { return Pre{}; }
   __device__ static void epilogue(const Op& op, int r, const typename Op::Acc& a, const Pre&, double* part) {
     op.epilogue_pre(r, a, op.prefetch(r), part);
+  }
+  __device__ static typename Op::GT epilogue_val(const Op& op, int r, const typename Op::Acc& a, const Pre&,
+                                                 double* part) {
+    return op.epilogue_pre(r, a, op.prefetch(r), part);
   }
 #endif
 };
@@ -872,12 +887,14 @@ struct PrimalOp {
     double c, l, u, x, sx, tau;
   };
   __device__ Pre prefetch(int j) const { return Pre{md.chat[j], md.lhat[j], md.uhat[j], w.x[j], w.sum_x[j], S->tau}; }
-  __device__ void epilogue_pre(int j, const Acc& a, const Pre& p, double*) const {
+  __device__ GT epilogue_pre(int j, const Acc& a, const Pre& p, double*) const {
     const double g = p.c - a.v[0];
     const double xn = clamp_i(p.x - p.tau * g, p.l, p.u);
-    w.xbar[j] = 2.0 * xn - p.x;
+    const double xb = 2.0 * xn - p.x;
+    w.xbar[j] = xb;
     w.sum_x[j] = p.sx + xn;
     w.x[j] = xn;
+    return xb;
   }
 };
 
@@ -903,12 +920,13 @@ struct DualOp {
     int8_t ge;
   };
   __device__ Pre prefetch(int i) const { return Pre{md.bhat[i], w.y[i], w.sum_y[i], S->sigma, md.ge[i]}; }
-  __device__ void epilogue_pre(int i, const Acc& a, const Pre& p, double*) const {
+  __device__ GT epilogue_pre(int i, const Acc& a, const Pre& p, double*) const {
     double yn = p.y + p.sigma * (p.b - a.v[0]);
     // y >= 0 on '>' rows (sign bit test); y = 0 on a row whose dual is fixed
     if (p.ge && (p.ge == kRowDualZero || __double_as_longlong(yn) < 0)) yn = 0.0;
     w.sum_y[i] = p.sy + yn;
     w.y[i] = yn;
+    return yn;
   }
 };
 
@@ -1047,7 +1065,7 @@ struct PrimalOpHT {
     const bool last = probe || it == last_it || S->k + it + 1 == S->max_iters;
     return Pre{md.chat[j], md.lhat[j], md.uhat[j], w.x[j], w.x_r[j], S->tau, h.hw[it], kUnitRho ? 1.0 : S->rho, last};
   }
-  __device__ void epilogue_pre(int j, const Acc& a, const Pre& p, double*) const {
+  __device__ GT epilogue_pre(int j, const Acc& a, const Pre& p, double*) const {
     const double g = p.c - a.v[0];
     const double xn = clamp_i(p.x - p.tau * g, p.l, p.u);
     const double xb = 2.0 * xn - p.x;
@@ -1061,6 +1079,7 @@ struct PrimalOpHT {
       h.xp[j] = xn;
       h.dx[j] = p.x - xn;
     }
+    return xb;
   }
 };
 using PrimalOpH = PrimalOpHT<false>;
@@ -1092,17 +1111,20 @@ struct DualOpHT {
     const bool last = probe || it == last_it || S->k + it + 1 == S->max_iters;
     return Pre{md.bhat[i], w.y[i], w.y_r[i], S->sigma, h.hw[it], kUnitRho ? 1.0 : S->rho, md.ge[i], last};
   }
-  __device__ void epilogue_pre(int i, const Acc& a, const Pre& p, double*) const {
+  __device__ GT epilogue_pre(int i, const Acc& a, const Pre& p, double*) const {
     double yn = p.y + p.sigma * (p.b - a.v[0]);
     if (p.ge && (p.ge == kRowDualZero || __double_as_longlong(yn) < 0)) yn = 0.0;
+    double yo = p.y;
     if (!probe) {
       const double r = (kUnitRho || p.rho == 1.0) ? fma(2.0, yn, -p.y) : fma(p.rho, yn - p.y, yn);
-      w.y[i] = fma(p.wt, r - p.y0, p.y0);
+      yo = fma(p.wt, r - p.y0, p.y0);
+      w.y[i] = yo;
     }
     if (p.last) {
       h.yp[i] = yn;
       h.dy[i] = p.y - yn;
     }
+    return yo;
   }
 };
 using DualOpH = DualOpHT<false>;
@@ -1437,6 +1459,12 @@ struct SumFF {
     r.lo[0] = __shfl_xor_sync(mask, lo[0], off);
     return r;
   }
+  __device__ __forceinline__ SumFF shfl_down(unsigned mask, int off) const {
+    SumFF r;
+    r.hi[0] = __shfl_down_sync(mask, hi[0], off);
+    r.lo[0] = __shfl_down_sync(mask, lo[0], off);
+    return r;
+  }
   __device__ __forceinline__ double value() const { return (double)hi[0] + (double)lo[0]; }
 };
 
@@ -1535,7 +1563,7 @@ struct PrimalOp32 {
   __device__ Pre prefetch(int j) const {
     return Pre{md.chat[j], md.lhat[j], md.uhat[j], w.x[j], w.xlo[j], (float)S->tau, w.sum_x[j]};
   }
-  __device__ void epilogue_pre(int j, const Acc& a, const Pre& p, double*) const {
+  __device__ GT epilogue_pre(int j, const Acc& a, const Pre& p, double*) const {
     // g = c - (A'y) from the float-float row sum: c - hi is exact when the two
     // are close (Sterbenz), so g keeps its relative precision near optimality
     const float g = (p.c - a.hi[0]) - a.lo[0];
@@ -1547,12 +1575,14 @@ struct PrimalOp32 {
       xh = xc;
       xl = 0.0f;
     }
-    w.xbar[j] = 2.0f * xh - p.x;
+    const float xb = 2.0f * xh - p.x;
+    w.xbar[j] = xb;
     float2 sx = p.sx;
     ff_add(sx, xh, xl);
     w.sum_x[j] = sx;
     w.x[j] = xh;
     w.xlo[j] = xl;
+    return xb;
   }
 };
 
@@ -1581,7 +1611,7 @@ struct DualOp32 {
   __device__ Pre prefetch(int i) const {
     return Pre{md.bhat[i], w.y[i], w.ylo[i], (float)S->sigma, md.ge[i], w.sum_y[i]};
   }
-  __device__ void epilogue_pre(int i, const Acc& a, const Pre& p, double*) const {
+  __device__ GT epilogue_pre(int i, const Acc& a, const Pre& p, double*) const {
     const float r = (p.b - a.hi[0]) - a.lo[0];
     float yh = p.y, yl = p.yl;
     ff_axpy(yh, yl, p.sigma, r);
@@ -1595,6 +1625,7 @@ struct DualOp32 {
     w.sum_y[i] = sy;
     w.y[i] = yh;
     w.ylo[i] = yl;
+    return yh;
   }
 };
 
@@ -1755,7 +1786,7 @@ struct PrimalOpH32T {
     return Pre{md.lhat[j], md.uhat[j], w.x[j], w.xlo[j], (float)S->tau, h.hs[it], (float)S->rho, w.q[j],
                w.xa[j], last};
   }
-  __device__ void epilogue_pre(int j, const Acc& a, const Pre& p, double*) const {
+  __device__ GT epilogue_pre(int j, const Acc& a, const Pre& p, double*) const {
     // g = c_hat - A_hat' y = q - A_hat' gy
     const float g = (p.q.x - a.hi[0]) + (p.q.y - a.lo[0]);
     float th = p.x, tl = p.xl;
@@ -1792,6 +1823,7 @@ struct PrimalOpH32T {
       h.xp[j] = (double)th + (double)tl;
       h.dx[j] = -((double)dh + (double)dl);
     }
+    return eh + el;
   }
 };
 using PrimalOpH32 = PrimalOpH32T<false>;
@@ -1822,7 +1854,7 @@ struct DualOpH32 {
     const bool last = probe || it == last_it || S->k + it + 1 == S->max_iters;
     return Pre{w.y[i], w.ylo[i], (float)S->sigma, h.hs[it], (float)S->rho, w.r0[i], w.ya[i], md.ge[i], last};
   }
-  __device__ void epilogue_pre(int i, const Acc& a, const Pre& p, double*) const {
+  __device__ GT epilogue_pre(int i, const Acc& a, const Pre& p, double*) const {
     // r = b_hat - A_hat x_bar = r0 - A_hat gx
     const float r = (p.r0.x - a.hi[0]) + (p.r0.y - a.lo[0]);
     float th = p.y, tl = p.yl;
@@ -1841,13 +1873,15 @@ struct DualOpH32 {
     // the next primal pass gathers the new y as its difference from the anchor
     float eh, el;
     ff_sub(yh, yl, p.y0.x, p.y0.y, eh, el);
-    w.gy[i] = eh + el;
+    const float gy = eh + el;
+    w.gy[i] = gy;
     if (p.last) {
       float dh, dl;
       ff_sub(p.y, p.yl, th, tl, dh, dl);
       h.yp[i] = (double)th + (double)tl;
       h.dy[i] = (double)dh + (double)dl;
     }
+    return gy;
   }
 };
 

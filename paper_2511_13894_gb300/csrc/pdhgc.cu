@@ -7,6 +7,7 @@
 // random-gather probe.
 #include <cuda_runtime.h>
 
+#include <algorithm>
 #include <chrono>
 #include <cmath>
 #include <cstdio>
@@ -14,11 +15,14 @@
 #include <cstring>
 #include <memory>
 #include <string>
+#include <utility>
 #include <vector>
 
 #include "../../include/pdhgc.h"
 #include "host_prep.h"
 #include "kernels.cuh"
+#include "steps.cuh"
+#include "batch.h"
 #include "guide.h"
 #include "kkt_eval.h"
 
@@ -55,11 +59,19 @@ int set_err(int code, const std::string& d) { return set_error_detail(code, d); 
       return set_err(PDHGC_ERR_CUDA, std::string("kernel launch: ") + cudaGetErrorString(e_)); \
   } while (0)
 
+#define RET(x)                 \
+  do {                         \
+    int r_ = (x);              \
+    if (r_ != PDHGC_OK) return r_; \
+  } while (0)
+
 // ---- report as computed on the device ------------------------------------
 struct DevReport {
   double rP2, rD2, rPinf, rDinf, pobj, dobj, gap, rel_p, rel_d, rel_gap, rel_kkt;
   double p, d, cand;
 };
+
+constexpr int kStepBar = 32;  // the barrier counter's place in step_seq (a line of its own)
 
 // ---- small kernels ---------------------------------------------------------
 
@@ -245,8 +257,10 @@ struct PhaseInit {
   double omega0;  // > 0: the starting primal weight (corner omega_rule 1); else from ||c_hat|| / ||b_hat||
 };
 
-__global__ void k_init_scalars(Scalars* S, PhaseInit pi, const double* cc2) {
+__global__ void k_init_scalars(Scalars* S, PhaseInit pi, const double* cc2, unsigned* seq) {
   if (threadIdx.x != 0) return;
+  seq[kStepBar] = 0u;
+  seq[0] += 1u;  // no step has number 0
   S->eps_rel = pi.eps_rel;
   S->beta_suff = pi.beta_suff;
   S->beta_nec = pi.beta_nec;
@@ -313,9 +327,17 @@ __global__ void k_h32_to64(const Scalars* S, int n, int m, const float* __restri
   if (i < m) y[i] = (double)y32[i] + (double)ylo[i];
 }
 
-// after a chunk of iterations: iteration counters and 1/t for the averages
-__global__ void k_pre_check(Scalars* S) {
+// after a chunk of iterations: iteration counters and 1/t for the averages; a
+// step kernel whose wait ran out (err) ends the phase.  seq: the step kernel's
+// counters (the next chunk's first step, its barrier)
+__global__ void k_pre_check(Scalars* S, unsigned* seq, const int* err) {
   if (threadIdx.x != 0 || S->done) return;
+  seq[0] += (unsigned)S->check_period;
+  seq[kStepBar] = 0u;
+  if (*err) {
+    S->done = 1;
+    return;
+  }
   long long run = S->max_iters - S->k;
   if (run > S->check_period) run = S->check_period;
   if (run < 0) run = 0;
@@ -707,6 +729,28 @@ struct pdhgc_lp {
     double* val64 = nullptr;
     float* val32 = nullptr;
   } ch64, ch32;
+  // the persistent step kernel (steps.cuh): a layout of A and A' per precision
+  struct StepSide {
+    StepTask* tasks = nullptr;
+    StepEpi* epis = nullptr;
+    StepSrcMap* map = nullptr;
+    int *warp_ptr = nullptr, *epi_ptr = nullptr, *slot_ptr = nullptr, *slot0 = nullptr, *col = nullptr;
+    void* val = nullptr;  // double (FP64) or float (FP32 bulk)
+    int ntasks = 0, max_tasks = 0, max_epis = 0, max_part = 0, max_slots = 0;
+  };
+  struct Steps {
+    bool on = false;  // runs the loop in this precision (else the per-pass kernels do)
+    StepSide A, T;
+    int hot_x = 0, hot_y = 0;
+    size_t smem = 0;
+    // (value, step) entries of x_bar and y; of this precision only: bits of the other's values would be read as steps
+    void *fx = nullptr, *fy = nullptr;
+  } steps64, steps32;
+  bool step_flow = false;
+  int step_ctas = 0;
+  size_t step_smem_max = 0;
+  unsigned* step_seq = nullptr;  // [0] step number of the next launch, [kStepBar] barrier arrivals
+  double* step_part = nullptr;   // 2 x ctas partial sums of the power iteration
   int chunked_primal = 0;  // 1: the Halpern loop's primal pass runs chunked (pdhgc_set_primal_layout)
   bool chunk_ready = false;  // the chunk plans are built on the first request for the chunked layout
   int launch_mode = PDHGC_LAUNCH_GRAPH;  // pdhgc_set_launch_mode
@@ -862,6 +906,151 @@ int launch_primal(pdhgc_lp* lp, const Op& op, cudaStream_t st, bool pdl) {
   return launch_tiles(lp, true, true, op, nullptr, st, pdl);
 }
 
+// ---- the persistent step kernel (steps.cuh) --------------------------------
+
+template <class VT>
+StepMat<VT> steps_side(const pdhgc_lp::StepSide& q) {
+  return StepMat<VT>{static_cast<const VT*>(q.val), q.col,       q.tasks,    q.epis,     q.warp_ptr, q.epi_ptr,
+                     q.slot_ptr,                    q.max_tasks, q.max_epis, q.max_part, q.max_slots};
+}
+
+StepFlow steps_flow(const pdhgc_lp* lp, const pdhgc_lp::Steps& sp) {
+  return StepFlow{sp.fy, sp.fx, lp->step_seq, lp->step_seq + kStepBar, lp->err, sp.hot_y, sp.hot_x};
+}
+
+// a cooperative launch of the step CTAs; the limit on dynamic shared memory is
+// always set to the same value, so that threads with other handles agree on it
+template <class... Par, class... Arg>
+int launch_coop(pdhgc_lp* lp, void (*kern)(Par...), size_t smem, cudaStream_t st, Arg&&... arg) {
+  CK(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)lp->step_smem_max));
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(lp->step_ctas);
+  cfg.blockDim = dim3(kStepThreads);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = st;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeCooperative;
+  attr[0].val.cooperative = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  CK(cudaLaunchKernelEx(&cfg, kern, std::forward<Arg>(arg)...));
+  lp->launches++;
+  return PDHGC_OK;
+}
+
+// all steps of a chunk (which = 3), or one of the two passes of each step
+template <class OpT, class OpA>
+int launch_steps(pdhgc_lp* lp, const OpT& opT, const OpA& opA, int period, int which, cudaStream_t st) {
+  using VT = typename OpT::VT;
+  const pdhgc_lp::Steps& sp = std::is_same<VT, float>::value ? lp->steps32 : lp->steps64;
+  const StepMat<VT> T = steps_side<VT>(sp.T), A = steps_side<VT>(sp.A);
+  const StepFlow flow = steps_flow(lp, sp);
+  return lp->step_flow ? launch_coop(lp, k_steps<true, OpT, OpA>, sp.smem, st, T, A, opT, opA, flow, period, which)
+                       : launch_coop(lp, k_steps<false, OpT, OpA>, sp.smem, st, T, A, opT, opA, flow, period, which);
+}
+
+// the loop of this precision and algorithm runs on the step kernel
+bool use_steps(const pdhgc_lp* lp, bool fp32, bool halpern) {
+  return (fp32 ? lp->steps32.on : lp->steps64.on) && !(halpern && lp->chunked_primal);
+}
+
+// the indices (once) or the values of a step layout, from the scaled CSR
+template <class VT>
+int fill_steps(pdhgc_lp* lp, const pdhgc_lp::Steps& sp, bool indices, cudaStream_t st) {
+  for (int t = 0; t < 2; ++t) {
+    const pdhgc_lp::StepSide& q = t ? sp.T : sp.A;
+    const pdhgc_lp::Mat& M = t ? lp->T : lp->A;
+    k_step_fill<VT><<<grid_for((long long)q.ntasks * 32), 256, 0, st>>>(
+        q.tasks, q.map, q.slot0, q.ntasks, M.rp, M.col, M.hat, indices ? q.col : nullptr,
+        indices ? nullptr : static_cast<VT*>(q.val));
+    lp->launches++;
+    CKL();
+  }
+  return PDHGC_OK;
+}
+
+// Plans and uploads the step layouts.  The step kernel runs an LP whose matrix
+// entries fit in the SMs' shared memory.  Measured (GB300, us per iteration, two
+// launches -> step kernel): power law, FP64, 0.32M nonzeros 16.3 -> 11.3; 1.25M,
+// the last to fit, 26.8 -> 26.7; FP32 0.32M 15.2 -> 12.4, 1.25M 24.6 -> 16.8;
+// without room for the entries it lost at 2.2M (FP64 31.3 -> 41.5, FP32 28.1 ->
+// 36.1): there the launches of many warps hide more latency than 16 warps a SM.
+// Flow order where no row is hot, and up to kFlowMaxNnz nonzeros with hot rows:
+// above, copying the hot entries costs more than the barriers (5000 x 20000
+// power law, 0.16M: barrier 8.6, flow 9.5; 2000 x 8000, 0.06M: 8.1 and 6.8-8.9).
+constexpr int64_t kFlowMaxNnz = 65536;
+constexpr int kStepCtaNnz = 128;  // at least this many nonzeros per CTA: small LPs leave SMs to other handles
+
+template <class VT>
+int setup_steps_one(pdhgc_lp* lp, pdhgc_lp::Steps& sp, const Csr& A, const Csr& T, cudaStream_t st) {
+  StepPlan plan[2];
+  plan_steps(A, lp->step_ctas, std::is_same<VT, float>::value, plan[0]);
+  plan_steps(T, lp->step_ctas, std::is_same<VT, float>::value, plan[1]);
+  if (!plan[0].ok || !plan[1].ok) return PDHGC_OK;
+  lp->step_flow = (plan[0].hot == 0 && plan[1].hot == 0) || lp->nnz <= kFlowMaxNnz;
+  sp.hot_y = lp->step_flow ? plan[0].hot : 0;
+  sp.hot_x = lp->step_flow ? plan[1].hot : 0;
+  sp.smem = sizeof(VT) * (size_t)(sp.hot_x + sp.hot_y);
+  for (const StepPlan& P : plan)
+    sp.smem += sizeof(StepTask) * (size_t)P.max_tasks + sizeof(StepEpi) * (size_t)P.max_epis +
+               2 * 8 * (size_t)P.max_part + (sizeof(VT) + sizeof(int)) * (size_t)P.max_slots;
+  if (sp.smem > lp->step_smem_max) return PDHGC_OK;
+  for (int t = 0; t < 2; ++t) {
+    pdhgc_lp::StepSide& q = t ? sp.T : sp.A;
+    const StepPlan& P = plan[t];
+    q.ntasks = (int)P.tasks.size();
+    q.max_tasks = P.max_tasks;
+    q.max_epis = P.max_epis;
+    q.max_part = P.max_part;
+    q.max_slots = P.max_slots;
+    auto up = [&](auto** dst, const auto& v) -> int {
+      RET(lp->alloc(dst, v.size()));
+      if (!v.empty()) CK(cudaMemcpyAsync(*dst, v.data(), v.size() * sizeof(v[0]), cudaMemcpyHostToDevice, st));
+      return PDHGC_OK;
+    };
+    RET(up(&q.tasks, P.tasks));
+    RET(up(&q.epis, P.epis));
+    RET(up(&q.map, P.map));
+    RET(up(&q.warp_ptr, P.warp_ptr));
+    RET(up(&q.epi_ptr, P.epi_ptr));
+    RET(up(&q.slot_ptr, P.slot_ptr));
+    RET(up(&q.slot0, P.slot0));
+    RET(lp->alloc(&q.col, (size_t)P.nslots));
+    VT* val;
+    RET(lp->alloc(&val, (size_t)P.nslots));
+    q.val = val;
+  }
+  if (lp->step_flow) {
+    const size_t entry = sizeof(typename StepEntry<VT>::type);
+    unsigned char *fx, *fy;
+    RET(lp->alloc(&fx, entry * (size_t)lp->n));
+    RET(lp->alloc(&fy, entry * (size_t)lp->m));
+    CK(cudaMemsetAsync(fx, 0, entry * (size_t)lp->n, st));
+    CK(cudaMemsetAsync(fy, 0, entry * (size_t)lp->m, st));
+    sp.fx = fx;
+    sp.fy = fy;
+  }
+  RET(fill_steps<VT>(lp, sp, true, st));
+  CK(cudaStreamSynchronize(st));  // the plans go out of scope
+  sp.on = true;
+  return PDHGC_OK;
+}
+
+int setup_steps(pdhgc_lp* lp, const Csr& A, const Csr& T, cudaStream_t st) {
+  int dev = 0, sms = 0, smem = 0, coop = 0;
+  CK(cudaGetDevice(&dev));
+  CK(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
+  CK(cudaDeviceGetAttribute(&smem, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev));
+  CK(cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, dev));
+  lp->step_smem_max = (size_t)smem - 1024;
+  const double room = (double)sms * (double)lp->step_smem_max;
+  if (!coop || 16.0 * (double)lp->nnz > room) return PDHGC_OK;
+  lp->step_ctas = (int)std::min<int64_t>(sms, std::max<int64_t>(1, lp->nnz / kStepCtaNnz));
+  RET(lp->alloc(&lp->step_part, 2 * (size_t)lp->step_ctas));
+  if (24.0 * (double)lp->nnz <= room) RET(setup_steps_one<double>(lp, lp->steps64, A, T, st));
+  return setup_steps_one<float>(lp, lp->steps32, A, T, st);
+}
+
 DevModel model_orig(const pdhgc_lp* lp) {
   return DevModel{lp->chat, lp->lhat, lp->uhat, lp->bhat, lp->Dr, lp->Dc, lp->ge};
 }
@@ -874,12 +1063,6 @@ DevModel32 model32_corner(const pdhgc_lp* lp) {
 DevModel model_corner(const pdhgc_lp* lp) {
   return DevModel{lp->chat_c, lp->lhat_c, lp->uhat_c, lp->bhat, lp->Dr, lp->Dc, lp->ge_c};
 }
-
-#define RET(x)                 \
-  do {                         \
-    int r_ = (x);              \
-    if (r_ != PDHGC_OK) return r_; \
-  } while (0)
 
 int to32(pdhgc_lp* lp, const double* a, float* b, long long n, cudaStream_t st) {
   if (n <= 0) return PDHGC_OK;
@@ -930,6 +1113,7 @@ int convert_fp32(pdhgc_lp* lp, cudaStream_t st) {
   RET(to32(lp, lp->lhat, lp->lhat32, lp->n, st));
   RET(to32(lp, lp->uhat, lp->uhat32, lp->n, st));
   RET(to32(lp, lp->bhat, lp->bhat32, lp->m, st));
+  if (lp->steps32.on) RET(fill_steps<float>(lp, lp->steps32, false, st));
   if (lp->ch32.nslots > 0) {  // the chunked pass's FP32 slots
     k_sell_fill<<<grid_for(lp->ch32.nslots), 256, 0, st>>>(lp->ch32.map, lp->T.hat32, lp->ch32.val32,
                                                           (int)lp->ch32.nslots);
@@ -973,6 +1157,7 @@ int setup_scaling(pdhgc_lp* lp, const pdhgc_params& p) {
                                                           (int)lp->ch64.nslots);
     lp->launches++;
   }
+  if (lp->steps64.on) RET(fill_steps<double>(lp, lp->steps64, false, st));
   k_scale_vectors<<<grid_for(m > n ? m : n), 256, 0, st>>>(m, n, lp->Dr, lp->Dc, lp->b_int, lp->c, lp->l,
                                                             lp->u, lp->bhat, lp->chat, lp->lhat, lp->uhat);
   k_norm2<<<1, 1024, 0, st>>>(lp->bhat, m, lp->scratch + 0);
@@ -983,6 +1168,17 @@ int setup_scaling(pdhgc_lp* lp, const pdhgc_params& p) {
   CK(cudaMemsetAsync(&lp->S->pi_zero, 0, sizeof(int), st));
   k_fill<<<grid_for(n), 256, 0, st>>>(lp->pi_v, n, 1.0 / std::sqrt((double)n));
   lp->launches++;
+  if (lp->steps64.on) {
+    const pdhgc_lp::Steps& sp = lp->steps64;
+    double* const part = lp->step_part + lp->step_ctas;
+    CK(cudaMemsetAsync(lp->step_seq + kStepBar, 0, sizeof(unsigned), st));
+    RET(launch_coop(lp, k_power, sp.smem, st, steps_side<double>(sp.T), steps_side<double>(sp.A), lp->S, lp->pi_v,
+                    lp->pi_u, lp->pi_w, lp->step_part, part, steps_flow(lp, sp), p.power_iters));
+    k_pi_final<<<1, 1024, 0, st>>>(lp->S, part, lp->step_ctas, p.eta_factor, lp->scratch + 0, lp->scratch + 1);
+    lp->launches++;
+    CKL();
+    return PDHGC_OK;
+  }
   for (int k = 0; k < p.power_iters; ++k) {
     RET(launch_tiles(lp, false, true, SpmvOp<false>{lp->S, lp->pi_v, lp->pi_u}, nullptr, st));
     RET(launch_tiles(lp, true, true, SpmvOp<true>{lp->S, lp->pi_u, lp->pi_w}, lp->pT, st));
@@ -1045,6 +1241,32 @@ int launch_anchor(pdhgc_lp* lp, const DevModel& md, int force, cudaStream_t st) 
   return PDHGC_OK;
 }
 
+// `count` steps of the loop by the step kernel (both passes, or one of them: launch_steps)
+int enqueue_steps(pdhgc_lp* lp, const DevModel& md, const DevModel32& md32, bool halpern, bool fp32, double rho,
+                  int count, int last, int which, cudaStream_t cs) {
+  const DevHalpern hz = lp->hz;
+  const DevIter w = lp->it;
+  if (halpern && fp32) {
+    const DualOpH32 d{lp->S, 0, last, 0, md32, h32_of(lp), hz};
+    return rho == 1.0
+               ? launch_steps(lp, PrimalOpH32T<true>{lp->S, 0, last, 0, md32, h32_of(lp), hz}, d, count, which, cs)
+               : launch_steps(lp, PrimalOpH32{lp->S, 0, last, 0, md32, h32_of(lp), hz}, d, count, which, cs);
+  }
+  if (halpern && rho == 1.0)
+    return launch_steps(lp, PrimalOpHT<true>{lp->S, 0, last, 0, w.y, md, w, hz},
+                        DualOpHT<true>{lp->S, 0, last, 0, w.xbar, md, w, hz}, count, which, cs);
+  if (halpern)
+    return launch_steps(lp, PrimalOpH{lp->S, 0, last, 0, w.y, md, w, hz}, DualOpH{lp->S, 0, last, 0, w.xbar, md, w, hz},
+                        count, which, cs);
+  if (fp32) {
+    const DevIter32 w32{lp->it32.x,   lp->it32.y,   lp->it32.xbar, lp->it32.sx, lp->it32.sy,
+                        lp->it32.xlo, lp->it32.ylo, lp->it32.xa,   lp->it32.ya};
+    return launch_steps(lp, PrimalOp32{lp->S, 0, lp->it32.y, md32, w32}, DualOp32{lp->S, 0, lp->it32.xbar, md32, w32},
+                        count, which, cs);
+  }
+  return launch_steps(lp, PrimalOp{lp->S, 0, w.y, md, w}, DualOp{lp->S, 0, w.xbar, md, w}, count, which, cs);
+}
+
 // Enqueues one loop body on `cs`: P iterations; pre-check; eval; decide;
 // restart; weights.  fp32 selects the FP32-bulk iteration kernels; the
 // evaluation and the decisions are FP64 in both.  use_handle: the decision
@@ -1059,7 +1281,10 @@ int enqueue_body(pdhgc_lp* lp, const DevModel& md, const DevModel32& md32, const
   const DevIter32 it32{lp->it32.x,  lp->it32.y,   lp->it32.xbar, lp->it32.sx, lp->it32.sy,
                        lp->it32.xlo, lp->it32.ylo, lp->it32.xa,   lp->it32.ya};
   int rc = PDHGC_OK;
-  for (int i = 0; i < pi.check_period && rc == PDHGC_OK; ++i) {
+  const bool persistent = use_steps(lp, fp32, halpern);
+  if (persistent)
+    rc = enqueue_steps(lp, md, md32, halpern, fp32, pi.rho, pi.check_period, pi.check_period - 1, 3, cs);
+  for (int i = 0; !persistent && i < pi.check_period && rc == PDHGC_OK; ++i) {
     if (halpern && fp32) {
       const int last = pi.check_period - 1;
       rc = pi.rho == 1.0 ? launch_primal(lp, PrimalOpH32T<true>{lp->S, i, last, 0, md32, h32_of(lp), hz}, cs, true)
@@ -1094,7 +1319,7 @@ int enqueue_body(pdhgc_lp* lp, const DevModel& md, const DevModel32& md32, const
     lp->launches++;
   }
   if (rc == PDHGC_OK) {
-    k_pre_check<<<1, 32, 0, cs>>>(lp->S);
+    k_pre_check<<<1, 32, 0, cs>>>(lp->S, lp->step_seq, lp->err);
     lp->launches++;
     rc = halpern ? launch_eval_h(lp, md, cs, ring) : launch_eval(lp, md, cs, ring);
   }
@@ -1187,7 +1412,7 @@ int run_phase(pdhgc_lp* lp, const DevModel& md, const DevModel32& md32, const Ph
   const DevIter32 it32{lp->it32.x,  lp->it32.y,   lp->it32.xbar, lp->it32.sx, lp->it32.sy,
                        lp->it32.xlo, lp->it32.ylo, lp->it32.xa,   lp->it32.ya};
   k_init_iterates<<<gnm, 256, 0, st>>>(n, m, md, lp->it, x_start, w32, y_start);
-  k_init_scalars<<<1, 32, 0, st>>>(lp->S, pi, cc2);
+  k_init_scalars<<<1, 32, 0, st>>>(lp->S, pi, cc2, lp->step_seq);
   lp->launches += 2;
   CKL();
   // phase 1 records its restart history (start point and restart points)
@@ -1235,6 +1460,7 @@ int run_phase(pdhgc_lp* lp, const DevModel& md, const DevModel32& md32, const Ph
   CK(cudaStreamSynchronize(st));
   int derr = 0;
   CK(cudaMemcpy(&derr, lp->err, sizeof(int), cudaMemcpyDeviceToHost));
+  if (derr != 0) CK(cudaMemset(lp->err, 0, sizeof(int)));  // reported once
   if (derr != 0) return set_err(PDHGC_ERR_DEVICE, "a bounded device wait ran out (error word " +
                                                       std::to_string(derr) + ")");
   return PDHGC_OK;
@@ -1912,6 +2138,15 @@ int pdhgc_lp_create(pdhgc_lp** out, int32_t m, int32_t n, int64_t nnz, const int
                     const int32_t* col_idx, const double* val, const double* b, const double* c,
                     const double* lb, const double* ub, const int8_t* sense, int inputs_on_device,
                     void* cuda_stream) {
+  return pdhgc::lp_create(out, m, n, nnz, row_ptr, col_idx, val, b, c, lb, ub, sense, inputs_on_device, cuda_stream,
+                          true);
+}
+
+}  // extern "C"
+
+int pdhgc::lp_create(pdhgc_lp** out, int32_t m, int32_t n, int64_t nnz, const int64_t* row_ptr,
+                     const int32_t* col_idx, const double* val, const double* b, const double* c, const double* lb,
+                     const double* ub, const int8_t* sense, int inputs_on_device, void* cuda_stream, bool own_gpu) {
   if (!out) return set_err(PDHGC_ERR_INVALID_ARG, "out is NULL");
   *out = nullptr;
   if (inputs_on_device != 0 && inputs_on_device != 1)
@@ -2033,11 +2268,16 @@ int pdhgc_lp_create(pdhgc_lp** out, int32_t m, int32_t n, int64_t nnz, const int
   CK(cudaMemcpyAsync(lp->row_perm, P.row_perm.data(), (size_t)m * 4, cudaMemcpyHostToDevice, st));
   CK(cudaMemcpyAsync(lp->col_perm, P.col_perm.data(), (size_t)n * 4, cudaMemcpyHostToDevice, st));
   CK(cudaMemsetAsync(lp->S, 0, sizeof(Scalars), st));
+  RET(lp->alloc(&lp->step_seq, kStepBar + 1));
+  CK(cudaMemsetAsync(lp->step_seq, 0, sizeof(unsigned) * (kStepBar + 1), st));
+  if (own_gpu) RET(setup_steps(lp.get(), P.A, P.AT, st));
   CK(cudaStreamSynchronize(st));  // the host vectors of P go out of scope
   pdhgc_default_params(&lp->params);
   *out = lp.release();
   return PDHGC_OK;
 }
+
+extern "C" {
 
 int pdhgc_solve(pdhgc_lp* lp, const pdhgc_params* params, pdhgc_report* out) {
   if (!lp) return set_err(PDHGC_ERR_INVALID_ARG, "lp is NULL");
@@ -2609,9 +2849,29 @@ int pdhgc_profile_iteration(pdhgc_lp* lp, int32_t iters, double* ms_out) {
   const long long big = (long long)1 << 62;
   CK(cudaMemcpy(&lp->S->done, &zero, sizeof(int), cudaMemcpyHostToDevice));
   CK(cudaMemcpy(&lp->S->max_iters, &big, sizeof(long long), cudaMemcpyHostToDevice));
-  std::vector<cudaEvent_t> ev(3 * (size_t)iters);
+  std::vector<cudaEvent_t> ev(3 * (size_t)iters + 1);
   for (auto& e : ev) CK(cudaEventCreate(&e));
   int rc = PDHGC_OK;
+  if (use_steps(lp, fp32, halpern)) {
+    // the step kernel: all primal passes in one launch, then all dual passes
+    for (int pass = 0; pass < 2 && rc == PDHGC_OK; ++pass) {
+      CK(cudaMemsetAsync(lp->step_seq + kStepBar, 0, sizeof(unsigned), st));
+      CK(cudaEventRecord(ev[2 * pass], st));
+      rc = enqueue_steps(lp, md, md32, halpern, fp32, lp->params.reflection, iters, 1, 1 << pass, st);
+      CK(cudaEventRecord(ev[2 * pass + 1], st));
+    }
+    CK(cudaMemsetAsync(lp->step_seq + kStepBar, 0, sizeof(unsigned), st));
+    CK(cudaStreamSynchronize(st));
+    for (int pass = 0; pass < 2 && rc == PDHGC_OK; ++pass) {
+      float ms = 0.f;
+      CK(cudaEventElapsedTime(&ms, ev[2 * pass], ev[2 * pass + 1]));
+      ms_out[pass] = ms / iters;
+    }
+    for (auto& e : ev) cudaEventDestroy(e);
+    CK(cudaMemcpy(&lp->S->done, &saved_done, sizeof(int), cudaMemcpyHostToDevice));
+    CK(cudaMemcpy(&lp->S->max_iters, &saved_max, sizeof(long long), cudaMemcpyHostToDevice));
+    return rc;
+  }
   for (int i = 0; i < iters && rc == PDHGC_OK; ++i) {
     CK(cudaEventRecord(ev[3 * i], st));
     // the Halpern loop's kernels as a step inside a chunk (it 0, not a check step)
