@@ -24,54 +24,89 @@ __device__ __forceinline__ double proj_dual_ev(double lam, double l, double u) {
   return 0.0;
 }
 
-// deterministic block fold of per-thread values into out (sum or max)
-__device__ double fold_block(double v, bool is_max, double* s_tmp) {
+// Per-block partials of NQ <= 8 quantities (a maximum where the bit of
+// kMaxMask is set), in a fixed order: the threads' values go through shared
+// memory and warp k folds quantity k.  An FP64 operation costs a scheduler 64
+// cycles whatever its active lanes, so 12 warp operations a quantity count
+// against the 104 of a shuffle tree in each of the 8 warps and an 8-term sum in
+// every thread.
+template <int NQ, unsigned kMaxMask>
+__device__ void fold_block(const double (&v)[NQ], double* __restrict__ part) {
+  static_assert(NQ <= kEvThreads / 32, "a warp per quantity");
+  __shared__ double s[NQ][kEvThreads];
+#pragma unroll
+  for (int k = 0; k < NQ; ++k) s[k][threadIdx.x] = v[k];
+  __syncthreads();
+  const int k = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  if (k >= NQ) return;
+  const bool is_max = (kMaxMask >> k) & 1u;
+  double x = s[k][lane];
+  for (int i = lane + 32; i < kEvThreads; i += 32) x = is_max ? fmax(x, s[k][i]) : x + s[k][i];
   for (int off = 16; off > 0; off >>= 1) {
-    const double o = __shfl_xor_sync(0xffffffffu, v, off);
-    v = is_max ? fmax(v, o) : v + o;
+    const double o = __shfl_xor_sync(0xffffffffu, x, off);
+    x = is_max ? fmax(x, o) : x + o;
   }
-  __syncthreads();
-  if ((threadIdx.x & 31) == 0) s_tmp[threadIdx.x >> 5] = v;
-  __syncthreads();
-  double t = s_tmp[0];
-  for (int w = 1; w < (int)(blockDim.x >> 5); ++w) t = is_max ? fmax(t, s_tmp[w]) : t + s_tmp[w];
-  return t;
+  if (lane == 0) part[k * kEvBlocks + blockIdx.x] = x;
 }
 
-__global__ void k_ev_zero(double* v, int n) {
-  for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) v[i] = 0.0;
-}
-
-// rows: (Ax)_i, the residual of each row under its sense, b'y, the slack
+// Rows: (Ax)_i, the residual of each row under its sense, b'y, the slack
 // metrics of inequality rows, and the scatter of y_i a_ij into A'y.
-// Partials (kEvRowQ per block): sum r^2, max |r|, sum b y, off, zero, cand.
-__global__ void __launch_bounds__(kEvThreads) k_ev_rows(EvalInput in, double* __restrict__ aty,
+// Partials (kEvRowQ per block): sum r^2, max |r|, sum b y, off, zero, cand,
+// sum b^2.  1 << lg lanes per row, 32 >> lg rows a warp at a time: the lane
+// reduction and the row's own operations are warp operations of the FP64 unit
+// shared by those rows; a row longer than kEvLong << lg is left to the whole
+// warp.  100k x 400k power law, 3.2M nonzeros, the whole evaluation: 996 us
+// with a warp per row, single-block norms and 1024 blocks folding with shuffles.
+constexpr int kEvLong = 64;
+__global__ void __launch_bounds__(kEvThreads) k_ev_rows(EvalInput in, int lg, double* __restrict__ aty,
                                                         double* __restrict__ part) {
-  __shared__ double s_tmp[32];
-  const int lane = threadIdx.x & 31;
+  const int lane = threadIdx.x & 31, L = 1 << lg, sub = lane & (L - 1);
+  const int rows_per = 32 >> lg;
   const int warps = gridDim.x * (blockDim.x >> 5);
-  double q[kEvRowQ] = {0, 0, 0, 0, 0, 0};
-  for (int i = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5); i < in.m; i += warps) {
-    const long long e0 = in.row_ptr[i], e1 = in.row_ptr[i + 1];
-    const double yi = in.y[i];
+  double q[kEvRowQ] = {0, 0, 0, 0, 0, 0, 0};
+  const long long groups = ((long long)in.m + rows_per - 1) / rows_per;
+  for (long long g = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5); g < groups; g += warps) {
+    const long long i = g * rows_per + (lane >> lg);
+    const bool has = i < in.m;
+    const long long e0 = has ? in.row_ptr[i] : 0, e1 = has ? in.row_ptr[i + 1] : 0;
+    const double yi = has ? in.y[i] : 0.0;
+    const bool is_long = e1 - e0 > (long long)kEvLong * L;
     double s = 0.0;
-    for (long long e = e0 + lane; e < e1; e += 32) {
-      const double a = in.val[e];
-      const int j = in.col_idx[e];
-      s = fma(a, in.x[j], s);
-      atomicAdd(aty + j, a * yi);
+    if (!is_long) {
+      for (long long e = e0 + sub; e < e1; e += L) {
+        const double a = in.val[e];
+        const int j = in.col_idx[e];
+        s = fma(a, in.x[j], s);
+        atomicAdd(aty + j, a * yi);
+      }
     }
-    for (int off = 16; off > 0; off >>= 1) s += __shfl_xor_sync(0xffffffffu, s, off);
-    if (lane == 0) {
+    for (int off = L >> 1; off > 0; off >>= 1) s += __shfl_xor_sync(0xffffffffu, s, off);
+    for (unsigned todo = __ballot_sync(0xffffffffu, is_long && sub == 0); todo; todo &= todo - 1) {
+      const int from = __ffs(todo) - 1;
+      const long long f0 = __shfl_sync(0xffffffffu, e0, from), f1 = __shfl_sync(0xffffffffu, e1, from);
+      const double yl = __shfl_sync(0xffffffffu, yi, from);
+      double t = 0.0;
+      for (long long e = f0 + lane; e < f1; e += 32) {
+        const double a = in.val[e];
+        const int j = in.col_idx[e];
+        t = fma(a, in.x[j], t);
+        atomicAdd(aty + j, a * yl);
+      }
+      for (int off = 16; off > 0; off >>= 1) t += __shfl_xor_sync(0xffffffffu, t, off);
+      if (lane == from) s = t;
+    }
+    if (has && sub == 0) {
       const char sn = in.sense ? (char)in.sense[i] : '=';
-      double r = in.b[i] - s;
+      const double bi = in.b[i];
+      double r = bi - s;
       if (sn == '<') r = fmin(r, 0.0);
       if (sn == '>') r = fmax(r, 0.0);
       q[0] += r * r;
       q[1] = fmax(q[1], fabs(r));
-      q[2] += in.b[i] * yi;
+      q[2] += bi * yi;
+      q[6] += bi * bi;
       if (sn != '=') {
-        const double slack = sn == '<' ? in.b[i] - s : s - in.b[i];
+        const double slack = sn == '<' ? bi - s : s - bi;
         const bool off = slack > 1e-6, zero = fabs(yi) <= 1e-6;
         q[3] += off ? 1.0 : 0.0;
         q[4] += zero ? 1.0 : 0.0;
@@ -79,63 +114,59 @@ __global__ void __launch_bounds__(kEvThreads) k_ev_rows(EvalInput in, double* __
       }
     }
   }
-  for (int k = 0; k < kEvRowQ; ++k) {
-    const double t = fold_block(q[k], k == 1, s_tmp);
-    if (threadIdx.x == 0) part[k * kEvBlocks + blockIdx.x] = t;
-  }
+  fold_block<kEvRowQ, 2u>(q, part);
 }
 
 // columns: lam = c - A'y, z = proj(lam), r_D = lam - z, c'x, the bound part
 // of the dual objective and the structural metrics.  Partials (kEvColQ per
-// block): sum r_D^2, max |r_D|, c x, l z+ - u z-, off, zero, cand.
+// block): sum r_D^2, max |r_D|, c x, l z+ - u z-, off, zero, cand, sum c^2.
 __global__ void __launch_bounds__(kEvThreads) k_ev_cols(EvalInput in, const double* __restrict__ aty,
                                                         double* __restrict__ part) {
-  __shared__ double s_tmp[32];
-  double q[kEvColQ] = {0, 0, 0, 0, 0, 0, 0};
+  double q[kEvColQ] = {0, 0, 0, 0, 0, 0, 0, 0};
   for (int j = blockIdx.x * blockDim.x + threadIdx.x; j < in.n; j += gridDim.x * blockDim.x) {
     const double l = in.lb ? in.lb[j] : 0.0;
     const double u = in.ub ? in.ub[j] : INFINITY;
-    const double lam = in.c[j] - aty[j];
+    const double cj = in.c[j];
+    const double lam = cj - aty[j];
     const double z = proj_dual_ev(lam, l, u);
     const double rd = lam - z;
     const double xj = in.x[j];
     q[0] += rd * rd;
     q[1] = fmax(q[1], fabs(rd));
-    q[2] += in.c[j] * xj;
+    q[2] += cj * xj;
     q[3] += (l != -INFINITY ? l * fmax(z, 0.0) : 0.0) - (u != INFINITY ? u * fmax(-z, 0.0) : 0.0);
     const bool off = fmin(xj - l, u - xj) > 1e-6, zero = fabs(z) <= 1e-6;
     q[4] += off ? 1.0 : 0.0;
     q[5] += zero ? 1.0 : 0.0;
     q[6] += (off && zero) ? 1.0 : 0.0;
+    q[7] += cj * cj;
   }
-  for (int k = 0; k < kEvColQ; ++k) {
-    const double t = fold_block(q[k], k == 1, s_tmp);
-    if (threadIdx.x == 0) part[k * kEvBlocks + blockIdx.x] = t;
-  }
+  fold_block<kEvColQ, 2u>(q, part);
 }
 
-// one CTA: fold the partials in block order and assemble the numbers
-__global__ void k_ev_final(const double* __restrict__ rpart, const double* __restrict__ cpart, double nb,
-                           double nc, double* __restrict__ out) {
-  __shared__ double s_tmp[32];
+// one CTA, a warp per quantity: fold the partials (lane t takes blocks t, t +
+// 32, ... in order) and assemble the numbers
+constexpr int kEvFinalThreads = 32 * (kEvRowQ + kEvColQ);
+__global__ void __launch_bounds__(kEvFinalThreads) k_ev_final(const double* __restrict__ rpart,
+                                                              const double* __restrict__ cpart,
+                                                              double* __restrict__ out) {
   __shared__ double q[kEvRowQ + kEvColQ];
-  for (int k = 0; k < kEvRowQ; ++k) {
-    double v = 0.0;
-    for (int b = threadIdx.x; b < kEvBlocks; b += blockDim.x)
-      v = k == 1 ? fmax(v, rpart[k * kEvBlocks + b]) : v + rpart[k * kEvBlocks + b];
-    const double t = fold_block(v, k == 1, s_tmp);
-    if (threadIdx.x == 0) q[k] = t;
+  const int k = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const double* p = k < kEvRowQ ? rpart + k * kEvBlocks : cpart + (k - kEvRowQ) * kEvBlocks;
+  const bool is_max = k == 1 || k == kEvRowQ + 1;
+  double v = 0.0;
+#pragma unroll 19
+  for (int b = lane; b < kEvBlocks; b += 32) v = is_max ? fmax(v, p[b]) : v + p[b];
+  for (int off = 16; off > 0; off >>= 1) {
+    const double o = __shfl_xor_sync(0xffffffffu, v, off);
+    v = is_max ? fmax(v, o) : v + o;
   }
-  for (int k = 0; k < kEvColQ; ++k) {
-    double v = 0.0;
-    for (int b = threadIdx.x; b < kEvBlocks; b += blockDim.x)
-      v = k == 1 ? fmax(v, cpart[k * kEvBlocks + b]) : v + cpart[k * kEvBlocks + b];
-    const double t = fold_block(v, k == 1, s_tmp);
-    if (threadIdx.x == 0) q[kEvRowQ + k] = t;
-  }
+  if (lane == 0) q[k] = v;
+  __syncthreads();
   if (threadIdx.x != 0) return;
   const double* c = q + kEvRowQ;
   const double rP2 = sqrt(q[0]), rD2 = sqrt(c[0]);
+  const double nb = sqrt(q[6]), nc = sqrt(c[7]);
   const double pobj = c[2], dobj = q[2] + c[3];
   out[0] = rP2;
   out[1] = rD2;
@@ -150,15 +181,6 @@ __global__ void k_ev_final(const double* __restrict__ rpart, const double* __res
   out[10] = q[3] + c[4];  // p
   out[11] = q[4] + c[5];  // d
   out[12] = q[5] + c[6];  // candidates
-}
-
-// ||v||_2^2 into out[0] (one CTA, fixed order)
-__global__ void k_ev_norm2(const double* __restrict__ v, int len, double* __restrict__ out) {
-  __shared__ double s_tmp[32];
-  double a = 0.0;
-  for (int i = threadIdx.x; i < len; i += blockDim.x) a += v[i] * v[i];
-  const double t = fold_block(a, false, s_tmp);
-  if (threadIdx.x == 0) out[0] = t;
 }
 
 }  // namespace
@@ -190,20 +212,18 @@ int kkt_eval_run(const EvalInput& in, double* scratch, cudaStream_t st, pdhgc_re
     detail = std::string(what) + ": " + cudaGetErrorString(e);
     return e == cudaErrorMemoryAllocation ? PDHGC_ERR_OOM : PDHGC_ERR_CUDA;
   };
-  k_ev_zero<<<kEvBlocks, kEvThreads, 0, st>>>(aty, in.n);
-  k_ev_rows<<<kEvBlocks, kEvThreads, 0, st>>>(in, aty, rpart);
+  cudaError_t e = cudaMemsetAsync(aty, 0, sizeof(double) * (size_t)in.n, st);
+  if (e != cudaSuccess) return fail(e, "kkt_eval clear");
+  // lanes per row: about 8 entries a lane of a mean row
+  int lg = 0;
+  while (lg < 5 && ((int64_t)in.m << (lg + 3)) < in.nnz) ++lg;
+  k_ev_rows<<<kEvBlocks, kEvThreads, 0, st>>>(in, lg, aty, rpart);
   k_ev_cols<<<kEvBlocks, kEvThreads, 0, st>>>(in, aty, cpart);
-  k_ev_norm2<<<1, kEvThreads, 0, st>>>(in.b, in.m, res + 13);
-  k_ev_norm2<<<1, kEvThreads, 0, st>>>(in.c, in.n, res + 14);
-  cudaError_t e = cudaGetLastError();
+  k_ev_final<<<1, kEvFinalThreads, 0, st>>>(rpart, cpart, res);
+  e = cudaGetLastError();
   if (e != cudaSuccess) return fail(e, "kkt_eval launch");
   double h[kEvOut];
-  e = cudaMemcpyAsync(h + 13, res + 13, 2 * sizeof(double), cudaMemcpyDeviceToHost, st);
-  if (e == cudaSuccess) e = cudaStreamSynchronize(st);
-  if (e != cudaSuccess) return fail(e, "kkt_eval norms");
-  k_ev_final<<<1, kEvThreads, 0, st>>>(rpart, cpart, std::sqrt(h[13]), std::sqrt(h[14]), res);
-  e = cudaGetLastError();
-  if (e == cudaSuccess) e = cudaMemcpyAsync(h, res, 13 * sizeof(double), cudaMemcpyDeviceToHost, st);
+  e = cudaMemcpyAsync(h, res, 13 * sizeof(double), cudaMemcpyDeviceToHost, st);
   if (e == cudaSuccess) e = cudaStreamSynchronize(st);
   if (e != cudaSuccess) return fail(e, "kkt_eval");
   std::memset(out, 0, sizeof(*out));
@@ -245,7 +265,7 @@ extern "C" int pdhgc_kkt_eval(int32_t m, int32_t n, int64_t nnz, const int64_t* 
   cudaError_t e = cudaMallocAsync(&scratch, bytes, st);
   if (e != cudaSuccess)
     return pdhgc::set_error_detail(PDHGC_ERR_OOM, std::string("cudaMallocAsync: ") + cudaGetErrorString(e));
-  pdhgc::EvalInput in{m, n, row_ptr, col_idx, val, b, c, lb, ub, sense, x, y};
+  pdhgc::EvalInput in{m, n, nnz, row_ptr, col_idx, val, b, c, lb, ub, sense, x, y};
   rc = pdhgc::kkt_eval_run(in, static_cast<double*>(scratch), st, out, detail);
   cudaFreeAsync(scratch, st);
   cudaStreamSynchronize(st);
@@ -329,7 +349,7 @@ extern "C" int pdhgc_kkt_eval_noalloc(int32_t m, int32_t n, int64_t nnz, const i
   double* scratch = nullptr;
   rc = scratch_for_current_device(&scratch, detail);
   if (rc != PDHGC_OK) return pdhgc::set_error_detail(rc, detail);
-  pdhgc::EvalInput in{m, n, row_ptr, col_idx, val, b, c, lb, ub, sense, x, y};
+  pdhgc::EvalInput in{m, n, nnz, row_ptr, col_idx, val, b, c, lb, ub, sense, x, y};
   rc = pdhgc::kkt_eval_run(in, scratch, static_cast<cudaStream_t>(cuda_stream), out, detail);
   if (rc != PDHGC_OK) return pdhgc::set_error_detail(rc, detail);
   return PDHGC_OK;

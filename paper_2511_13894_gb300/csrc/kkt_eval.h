@@ -10,14 +10,15 @@
 
 namespace pdhgc {
 
-constexpr int kEvBlocks = 1024;  // fixed grid: the reduction order does not depend on the GPU
+constexpr int kEvBlocks = 608;   // fixed grid (4 per SM of a GB300): the reduction order does not depend on the GPU
 constexpr int kEvThreads = 256;
-constexpr int kEvRowQ = 6;       // partial quantities per block from the rows
-constexpr int kEvColQ = 7;       // partial quantities per block from the columns
+constexpr int kEvRowQ = 7;       // partial quantities per block from the rows
+constexpr int kEvColQ = 8;       // partial quantities per block from the columns
 constexpr int kEvOut = 16;       // doubles of assembled results
 
 struct EvalInput {
   int m, n;
+  int64_t nnz;
   const int64_t* row_ptr;
   const int32_t* col_idx;
   const double* val;
