@@ -85,19 +85,41 @@ __device__ __forceinline__ unsigned long long mix64(unsigned long long seed, uns
   return z ^ (z >> 31);
 }
 
-// stage W1 (padded, stride 40) and W2 (stride 72) and optionally W2' in shared memory
+// stage W1 (padded, stride 40) and W2 (stride 72) and optionally W2' in shared
+// memory, 16 bytes a load: all of a thread's loads are in flight together (10
+// in the training kernel; one word each, 40 in batches, took several times
+// the latency of L2).  From L2: a training kernel may start before the update
+// of the weights it reads has ended, beside CTAs that hold the old ones in L1
 __device__ void stage_weights(const GuideBf16* __restrict__ wb, __nv_bfloat16* sW1, __nv_bfloat16* sW2,
                               __nv_bfloat16* sW2T) {
-  const uint32_t* w1 = reinterpret_cast<const uint32_t*>(wb->w1);
-  const uint32_t* w2 = reinterpret_cast<const uint32_t*>(wb->w2);
-  const uint32_t* w2t = reinterpret_cast<const uint32_t*>(wb->w2t);
-  uint32_t* s1 = reinterpret_cast<uint32_t*>(sW1);
-  uint32_t* s2 = reinterpret_cast<uint32_t*>(sW2);
-  uint32_t* s2t = reinterpret_cast<uint32_t*>(sW2T);
-  for (int e = threadIdx.x; e < kGHid * 16; e += blockDim.x) s1[(e >> 4) * (kS40 / 2) + (e & 15)] = w1[e];
-  for (int e = threadIdx.x; e < kGHid * 32; e += blockDim.x) {
-    s2[(e >> 5) * (kS72 / 2) + (e & 31)] = w2[e];
-    if (sW2T) s2t[(e >> 5) * (kS72 / 2) + (e & 31)] = w2t[e];
+  static_assert(kGFeat == 32 && kGHid == 64 && kS40 % 8 == 0 && kS72 % 8 == 0, "16-byte pieces of rows");
+  const uint4* w1 = reinterpret_cast<const uint4*>(wb->w1);
+  const uint4* w2 = reinterpret_cast<const uint4*>(wb->w2);
+  const uint4* w2t = reinterpret_cast<const uint4*>(wb->w2t);
+  uint4* s1 = reinterpret_cast<uint4*>(sW1);
+  uint4* s2 = reinterpret_cast<uint4*>(sW2);
+  uint4* s2t = reinterpret_cast<uint4*>(sW2T);
+  constexpr int N1 = kGHid * 4 / kGThreads, N2 = kGHid * 8 / kGThreads;
+  static_assert(N1 * kGThreads == kGHid * 4 && N2 * kGThreads == kGHid * 8, "whole pieces per thread");
+  const int tid = threadIdx.x;
+  uint4 v1[N1], v2[N2], v3[N2];
+#pragma unroll
+  for (int i = 0; i < N1; ++i) v1[i] = __ldcg(w1 + tid + i * kGThreads);
+#pragma unroll
+  for (int i = 0; i < N2; ++i) v2[i] = __ldcg(w2 + tid + i * kGThreads);
+  if (sW2T)
+#pragma unroll
+    for (int i = 0; i < N2; ++i) v3[i] = __ldcg(w2t + tid + i * kGThreads);
+#pragma unroll
+  for (int i = 0; i < N1; ++i) {
+    const int e = tid + i * kGThreads;
+    s1[(e >> 2) * (kS40 / 8) + (e & 3)] = v1[i];
+  }
+#pragma unroll
+  for (int i = 0; i < N2; ++i) {
+    const int e = tid + i * kGThreads;
+    s2[(e >> 3) * (kS72 / 8) + (e & 7)] = v2[i];
+    if (sW2T) s2t[(e >> 3) * (kS72 / 8) + (e & 7)] = v3[i];
   }
 }
 
@@ -491,11 +513,39 @@ __global__ void __launch_bounds__(kGThreads) k_guide_grad(const GuideBf16* __res
                                                            float* __restrict__ partials) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   TrainSmem& s = *reinterpret_cast<TrainSmem*>(smem_raw);
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, g = lane >> 2, t = lane & 3;
+  const uint32_t* f = reinterpret_cast<const uint32_t*>(feat);
+  uint32_t* sx = reinterpret_cast<uint32_t*>(s.x);
+  float lab = 0.0f;
+  // the warp's 16 samples of chunk c: dataset rows (staged) and labels
+  auto load_samples = [&](int c) {
+    const int s_base = c * kChunk + warp * 16;
+    long long src = -1;
+    lab = 0.0f;
+    if (lane < 16 && s_base + lane < batch) {
+      const int sidx = s_base + lane;
+      src = idx ? (long long)idx[sidx]
+                : (long long)(mix64(seed, (unsigned long long)step * (unsigned long long)batch + sidx) %
+                              (unsigned long long)rows);
+      lab = labels[src] ? 1.0f : 0.0f;
+    }
+#pragma unroll
+    for (int u = 0; u < 8; ++u) {
+      const int e = lane + 32 * u, rr = e >> 4, kw = e & 15;
+      const long long sr = __shfl_sync(0xffffffffu, src, rr);
+      sx[(warp * 16 + rr) * (kS40 / 2) + kw] = sr >= 0 ? f[sr * 16 + kw] : 0u;
+    }
+  };
+  // with programmatic dependent launch (the training loop): the samples do not
+  // depend on the previous step, the weights and the partials do
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  load_samples(blockIdx.x);
+  asm volatile("griddepcontrol.wait;" ::: "memory");
   stage_weights(wb, s.w1, s.w2, s.w2t);
   for (int j = threadIdx.x; j < kGHid; j += blockDim.x) {
-    s.b1[j] = w[kOffB1 + j];
-    s.b2[j] = w[kOffB2 + j];
-    s.w3[j] = __bfloat162float(wb->w3[j]);
+    s.b1[j] = __ldcg(w + kOffB1 + j);
+    s.b2[j] = __ldcg(w + kOffB2 + j);
+    s.w3[j] = __bfloat162float(__ldcg(wb->w3 + j));
     for (int q = 0; q < kGWarps; ++q) {
       s.gb1[q][j] = 0.0f;
       s.gb2[q][j] = 0.0f;
@@ -506,12 +556,9 @@ __global__ void __launch_bounds__(kGThreads) k_guide_grad(const GuideBf16* __res
     s.gb3[threadIdx.x] = 0.0f;
     s.loss[threadIdx.x] = 0.0f;
   }
-  const float b3 = w[kOffB3];
+  const float b3 = __ldcg(w + kOffB3);
   const float inv_b = 1.0f / (float)batch;
   __syncthreads();
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, g = lane >> 2, t = lane & 3;
-  const uint32_t* f = reinterpret_cast<const uint32_t*>(feat);
-  uint32_t* sx = reinterpret_cast<uint32_t*>(s.x);
   const uint32_t* sw2t = reinterpret_cast<const uint32_t*>(s.w2t);
   float gW2[8][4], gW1[4][4];
 #pragma unroll
@@ -520,22 +567,8 @@ __global__ void __launch_bounds__(kGThreads) k_guide_grad(const GuideBf16* __res
   for (int nt = 0; nt < 4; ++nt) gW1[nt][0] = gW1[nt][1] = gW1[nt][2] = gW1[nt][3] = 0.0f;
   const int nchunks = (batch + kChunk - 1) / kChunk;
   for (int c = blockIdx.x; c < nchunks; c += gridDim.x) {
-    // ---- the warp's 16 samples: dataset rows and labels
     const int s_base = c * kChunk + warp * 16;
-    long long src = -1;
-    float lab = 0.0f;
-    if (lane < 16 && s_base + lane < batch) {
-      const int sidx = s_base + lane;
-      src = idx ? (long long)idx[sidx]
-                : (long long)(mix64(seed, (unsigned long long)step * (unsigned long long)batch + sidx) %
-                              (unsigned long long)rows);
-      lab = labels[src] ? 1.0f : 0.0f;
-    }
-    for (int e = lane; e < 16 * 16; e += 32) {
-      const int rr = e >> 4, kw = e & 15;
-      const long long sr = __shfl_sync(0xffffffffu, src, rr);
-      sx[(warp * 16 + rr) * (kS40 / 2) + kw] = sr >= 0 ? f[sr * 16 + kw] : 0u;
-    }
+    if (c != (int)blockIdx.x) load_samples(c);
     const float y0 = __shfl_sync(0xffffffffu, lab, g), y1 = __shfl_sync(0xffffffffu, lab, g + 8);
     const bool v0 = s_base + g < batch, v1 = s_base + g + 8 < batch;
     __syncwarp();
@@ -725,27 +758,40 @@ __device__ __forceinline__ void write_bf16(GuideBf16* wb, int p, float v) {
   }
 }
 
+constexpr int kFoldBatch = 32;
+constexpr int kFoldThreads = 64;  // per CTA: the parameters spread over 87 SMs
 // fold the per-CTA partials in CTA order; lr > 0: one Adam step
 // (Kingma & Ba 2015, beta1 = 0.9, beta2 = 0.999, eps = 1e-8) with the bias
 // corrections c1 = 1 / (1 - beta1^t), c2 = 1 / (1 - beta2^t)
 __global__ void k_guide_fold(const float* __restrict__ partials, int nparts, float* __restrict__ grad,
                              float* __restrict__ w, float* __restrict__ m1, float* __restrict__ m2,
                              GuideBf16* __restrict__ wb, float lr, float c1, float c2, float* __restrict__ loss_hist) {
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   const int p = blockIdx.x * blockDim.x + threadIdx.x;
   if (p >= kGPartial) return;
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+  // in CTA order, kFoldBatch loads in flight (one after another, 64 partials
+  // cost 64 latencies of L2 in batches of 4)
   float gsum = 0.0f;
-  for (int b = 0; b < nparts; ++b) gsum += partials[(size_t)b * kGPartial + p];
+  for (int b0 = 0; b0 < nparts; b0 += kFoldBatch) {
+    float v[kFoldBatch];
+#pragma unroll
+    for (int u = 0; u < kFoldBatch; ++u) v[u] = __ldcg(partials + (size_t)min(b0 + u, nparts - 1) * kGPartial + p);
+#pragma unroll
+    for (int u = 0; u < kFoldBatch; ++u)
+      if (b0 + u < nparts) gsum += v[u];
+  }
   grad[p] = gsum;
   if (p == kGParams) {
     if (loss_hist) *loss_hist = gsum;
     return;
   }
   if (lr > 0.0f) {
-    const float a = 0.9f * m1[p] + 0.1f * gsum;
-    const float v = 0.999f * m2[p] + 0.001f * gsum * gsum;
+    const float a = 0.9f * __ldcg(m1 + p) + 0.1f * gsum;
+    const float v = 0.999f * __ldcg(m2 + p) + 0.001f * gsum * gsum;
     m1[p] = a;
     m2[p] = v;
-    const float wn = w[p] - lr * (a * c1) / (sqrtf(v * c2) + 1e-8f);
+    const float wn = __ldcg(w + p) - lr * (a * c1) / (sqrtf(v * c2) + 1e-8f);
     w[p] = wn;
     write_bf16(wb, p, wn);
   }
@@ -817,7 +863,7 @@ int guide_step(pdhgc_guide* g, const __nv_bfloat16* feat, const uint8_t* labels,
     c1 = (float)(1.0 / (1.0 - std::pow(0.9, (double)g->adam_t)));
     c2 = (float)(1.0 / (1.0 - std::pow(0.999, (double)g->adam_t)));
   }
-  k_guide_fold<<<(kGPartial + 255) / 256, 256, 0, st>>>(g->partials, grid, g->grad, g->w, g->m1, g->m2, g->wb,
+  k_guide_fold<<<(kGPartial + kFoldThreads - 1) / kFoldThreads, kFoldThreads, 0, st>>>(g->partials, grid, g->grad, g->w, g->m1, g->m2, g->wb,
                                                         adam_lr, c1, c2, nullptr);
   g->launches++;
   GKL();
@@ -1048,18 +1094,36 @@ int pdhgc_guide_train(pdhgc_guide* g, const uint16_t* feat, const uint8_t* label
   float* hist = nullptr;
   if (losses && steps > 0) GK(cudaMallocAsync(&hist, sizeof(float) * (size_t)steps, g->stream));
   for (int64_t s = 0; s < steps; ++s) {
+    // each kernel starts under the one before it (programmatic dependent
+    // launch; the first gradient kernel is ordered after the caller's work)
     const int nchunks = (batch + kChunk - 1) / kChunk;
     const int grid = nchunks < g->max_ctas ? nchunks : g->max_ctas;
-    k_guide_grad<<<grid, kGThreads, train_smem(), g->stream>>>(
-        g->wb, g->w, reinterpret_cast<const __nv_bfloat16*>(feat), labels, (long long)rows, nullptr, batch,
-        (unsigned long long)seed, (long long)s, g->partials);
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(grid);
+    cfg.blockDim = dim3(kGThreads);
+    cfg.dynamicSmemBytes = train_smem();
+    cfg.stream = g->stream;
+    cfg.attrs = attr;
+    cfg.numAttrs = s > 0 ? 1 : 0;
+    cudaError_t e = cudaLaunchKernelEx(&cfg, k_guide_grad, (const GuideBf16*)g->wb, (const float*)g->w,
+                                       reinterpret_cast<const __nv_bfloat16*>(feat), labels, (long long)rows,
+                                       (const int32_t*)nullptr, batch, (unsigned long long)seed, (long long)s,
+                                       g->partials);
     g->adam_t++;
     const float c1 = (float)(1.0 / (1.0 - std::pow(0.9, (double)g->adam_t)));
     const float c2 = (float)(1.0 / (1.0 - std::pow(0.999, (double)g->adam_t)));
-    k_guide_fold<<<(kGPartial + 255) / 256, 256, 0, g->stream>>>(g->partials, grid, g->grad, g->w, g->m1, g->m2,
-                                                                 g->wb, lr, c1, c2, hist ? hist + s : nullptr);
+    cfg.gridDim = dim3((kGPartial + kFoldThreads - 1) / kFoldThreads);
+    cfg.blockDim = dim3(kFoldThreads);
+    cfg.dynamicSmemBytes = 0;
+    cfg.numAttrs = 1;
+    if (e == cudaSuccess)
+      e = cudaLaunchKernelEx(&cfg, k_guide_fold, (const float*)g->partials, grid, g->grad, g->w, g->m1, g->m2, g->wb,
+                             lr, c1, c2, hist ? hist + s : (float*)nullptr);
+    if (e == cudaSuccess) e = cudaGetLastError();
     g->launches += 2;
-    cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) {
       if (hist) cudaFreeAsync(hist, g->stream);
       return set_error_detail(PDHGC_ERR_CUDA, std::string("guide train launch: ") + cudaGetErrorString(e));
