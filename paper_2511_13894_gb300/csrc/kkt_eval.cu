@@ -64,6 +64,7 @@ __global__ void __launch_bounds__(kEvThreads) k_ev_rows(EvalInput in, int lg, do
   const int rows_per = 32 >> lg;
   const int warps = gridDim.x * (blockDim.x >> 5);
   double q[kEvRowQ] = {0, 0, 0, 0, 0, 0, 0};
+  int n_off = 0, n_zero = 0, n_cand = 0;  // off the FP64 unit
   const long long groups = ((long long)in.m + rows_per - 1) / rows_per;
   for (long long g = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5); g < groups; g += warps) {
     const long long i = g * rows_per + (lane >> lg);
@@ -108,12 +109,15 @@ __global__ void __launch_bounds__(kEvThreads) k_ev_rows(EvalInput in, int lg, do
       if (sn != '=') {
         const double slack = sn == '<' ? bi - s : s - bi;
         const bool off = slack > 1e-6, zero = fabs(yi) <= 1e-6;
-        q[3] += off ? 1.0 : 0.0;
-        q[4] += zero ? 1.0 : 0.0;
-        q[5] += (off && zero) ? 1.0 : 0.0;
+        n_off += off;
+        n_zero += zero;
+        n_cand += off && zero;
       }
     }
   }
+  q[3] = n_off;
+  q[4] = n_zero;
+  q[5] = n_cand;
   fold_block<kEvRowQ, 2u>(q, part);
 }
 
@@ -123,6 +127,7 @@ __global__ void __launch_bounds__(kEvThreads) k_ev_rows(EvalInput in, int lg, do
 __global__ void __launch_bounds__(kEvThreads) k_ev_cols(EvalInput in, const double* __restrict__ aty,
                                                         double* __restrict__ part) {
   double q[kEvColQ] = {0, 0, 0, 0, 0, 0, 0, 0};
+  int n_off = 0, n_zero = 0, n_cand = 0;
   for (int j = blockIdx.x * blockDim.x + threadIdx.x; j < in.n; j += gridDim.x * blockDim.x) {
     const double l = in.lb ? in.lb[j] : 0.0;
     const double u = in.ub ? in.ub[j] : INFINITY;
@@ -136,11 +141,14 @@ __global__ void __launch_bounds__(kEvThreads) k_ev_cols(EvalInput in, const doub
     q[2] += cj * xj;
     q[3] += (l != -INFINITY ? l * fmax(z, 0.0) : 0.0) - (u != INFINITY ? u * fmax(-z, 0.0) : 0.0);
     const bool off = fmin(xj - l, u - xj) > 1e-6, zero = fabs(z) <= 1e-6;
-    q[4] += off ? 1.0 : 0.0;
-    q[5] += zero ? 1.0 : 0.0;
-    q[6] += (off && zero) ? 1.0 : 0.0;
+    n_off += off;
+    n_zero += zero;
+    n_cand += off && zero;
     q[7] += cj * cj;
   }
+  q[4] = n_off;
+  q[5] = n_zero;
+  q[6] = n_cand;
   fold_block<kEvColQ, 2u>(q, part);
 }
 
@@ -267,8 +275,10 @@ extern "C" int pdhgc_kkt_eval(int32_t m, int32_t n, int64_t nnz, const int64_t* 
     return pdhgc::set_error_detail(PDHGC_ERR_OOM, std::string("cudaMallocAsync: ") + cudaGetErrorString(e));
   pdhgc::EvalInput in{m, n, nnz, row_ptr, col_idx, val, b, c, lb, ub, sense, x, y};
   rc = pdhgc::kkt_eval_run(in, static_cast<double*>(scratch), st, out, detail);
+  // the evaluation has ended (its results were read): no synchronisation behind
+  // the free, at which the device's default pool would unmap the scratch and
+  // the next call map it again, 165 us of an evaluation of the 100k x 400k LP
   cudaFreeAsync(scratch, st);
-  cudaStreamSynchronize(st);
   if (rc != PDHGC_OK) return pdhgc::set_error_detail(rc, detail);
   return PDHGC_OK;
 }
