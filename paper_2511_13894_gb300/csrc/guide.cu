@@ -37,6 +37,7 @@ namespace {
 
 constexpr int kGWarps = 4;
 constexpr int kGThreads = kGWarps * 32;
+constexpr int kTrainSteps = 1024;      // steps per launch of the training kernel
 constexpr int kChunk = kGWarps * 16;  // samples per CTA step of the training kernel
 constexpr int kS40 = 40;               // padded shared row of 32 BF16 (conflict-free fragment loads)
 constexpr int kS72 = 72;               // padded shared row of 64 BF16
@@ -504,43 +505,48 @@ __device__ __forceinline__ void col_sums_add(float (&v)[8][2], float* acc) {
     }
 }
 
-__global__ void __launch_bounds__(kGThreads) k_guide_grad(const GuideBf16* __restrict__ wb,
-                                                           const float* __restrict__ w,
-                                                           const __nv_bfloat16* __restrict__ feat,
-                                                           const uint8_t* __restrict__ labels, long long rows,
-                                                           const int32_t* __restrict__ idx, int batch,
-                                                           unsigned long long seed, long long step,
-                                                           float* __restrict__ partials) {
-  extern __shared__ __align__(16) unsigned char smem_raw[];
-  TrainSmem& s = *reinterpret_cast<TrainSmem*>(smem_raw);
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, g = lane >> 2, t = lane & 3;
-  const uint32_t* f = reinterpret_cast<const uint32_t*>(feat);
+// what a gradient is taken of: `batch` dataset rows, given (idx) or drawn by
+// SplitMix64(seed, step * batch + sample) mod rows
+struct GuideBatch {
+  const __nv_bfloat16* feat;
+  const uint8_t* labels;
+  long long rows;
+  const int32_t* idx;
+  int batch;
+  unsigned long long seed;
+};
+
+// the warp's 16 samples of chunk c: features staged, the lane's label returned
+__device__ __forceinline__ float load_samples(TrainSmem& s, const GuideBatch& B, long long step, int c) {
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const uint32_t* f = reinterpret_cast<const uint32_t*>(B.feat);
   uint32_t* sx = reinterpret_cast<uint32_t*>(s.x);
+  const int s_base = c * kChunk + warp * 16;
+  long long src = -1;
   float lab = 0.0f;
-  // the warp's 16 samples of chunk c: dataset rows (staged) and labels
-  auto load_samples = [&](int c) {
-    const int s_base = c * kChunk + warp * 16;
-    long long src = -1;
-    lab = 0.0f;
-    if (lane < 16 && s_base + lane < batch) {
-      const int sidx = s_base + lane;
-      src = idx ? (long long)idx[sidx]
-                : (long long)(mix64(seed, (unsigned long long)step * (unsigned long long)batch + sidx) %
-                              (unsigned long long)rows);
-      lab = labels[src] ? 1.0f : 0.0f;
-    }
+  if (lane < 16 && s_base + lane < B.batch) {
+    const int sidx = s_base + lane;
+    src = B.idx ? (long long)B.idx[sidx]
+                : (long long)(mix64(B.seed, (unsigned long long)step * (unsigned long long)B.batch + sidx) %
+                              (unsigned long long)B.rows);
+    lab = B.labels[src] ? 1.0f : 0.0f;
+  }
 #pragma unroll
-    for (int u = 0; u < 8; ++u) {
-      const int e = lane + 32 * u, rr = e >> 4, kw = e & 15;
-      const long long sr = __shfl_sync(0xffffffffu, src, rr);
-      sx[(warp * 16 + rr) * (kS40 / 2) + kw] = sr >= 0 ? f[sr * 16 + kw] : 0u;
-    }
-  };
-  // with programmatic dependent launch (the training loop): the samples do not
-  // depend on the previous step, the weights and the partials do
-  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-  load_samples(blockIdx.x);
-  asm volatile("griddepcontrol.wait;" ::: "memory");
+  for (int u = 0; u < 8; ++u) {
+    const int e = lane + 32 * u, rr = e >> 4, kw = e & 15;
+    const long long sr = __shfl_sync(0xffffffffu, src, rr);
+    sx[(warp * 16 + rr) * (kS40 / 2) + kw] = sr >= 0 ? f[sr * 16 + kw] : 0u;
+  }
+  return lab;
+}
+
+// the CTA's partial gradient (and loss) of one step over its chunks
+// blockIdx.x, blockIdx.x + gridDim.x, ...; the first one's samples are loaded
+__device__ __forceinline__ void grad_cta(TrainSmem& s, const GuideBf16* __restrict__ wb, const float* __restrict__ w,
+                                         const GuideBatch& B, long long step, float lab, float* __restrict__ out) {
+  const int batch = B.batch;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, g = lane >> 2, t = lane & 3;
+  const uint32_t* sx = reinterpret_cast<const uint32_t*>(s.x);
   stage_weights(wb, s.w1, s.w2, s.w2t);
   for (int j = threadIdx.x; j < kGHid; j += blockDim.x) {
     s.b1[j] = __ldcg(w + kOffB1 + j);
@@ -568,7 +574,7 @@ __global__ void __launch_bounds__(kGThreads) k_guide_grad(const GuideBf16* __res
   const int nchunks = (batch + kChunk - 1) / kChunk;
   for (int c = blockIdx.x; c < nchunks; c += gridDim.x) {
     const int s_base = c * kChunk + warp * 16;
-    if (c != (int)blockIdx.x) load_samples(c);
+    if (c != (int)blockIdx.x) lab = load_samples(s, B, step, c);
     const float y0 = __shfl_sync(0xffffffffu, lab, g), y1 = __shfl_sync(0xffffffffu, lab, g + 8);
     const bool v0 = s_base + g < batch, v1 = s_base + g + 8 < batch;
     __syncwarp();
@@ -699,7 +705,6 @@ __global__ void __launch_bounds__(kGThreads) k_guide_grad(const GuideBf16* __res
     __syncthreads();
   }
   // ---- this CTA's partial gradient
-  float* out = partials + (size_t)blockIdx.x * kGPartial;
   const int j0 = warp * 16;
 #pragma unroll
   for (int nt = 0; nt < 8; ++nt) {
@@ -743,6 +748,15 @@ __global__ void __launch_bounds__(kGThreads) k_guide_grad(const GuideBf16* __res
   }
 }
 
+__global__ void __launch_bounds__(kGThreads) k_guide_grad(const GuideBf16* __restrict__ wb,
+                                                           const float* __restrict__ w, GuideBatch B, long long step,
+                                                           float* __restrict__ partials) {
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  TrainSmem& s = *reinterpret_cast<TrainSmem*>(smem_raw);
+  const float lab = load_samples(s, B, step, blockIdx.x);
+  grad_cta(s, wb, w, B, step, lab, partials + (size_t)blockIdx.x * kGPartial);
+}
+
 // BF16 copy of parameter p of the packed vector
 __device__ __forceinline__ void write_bf16(GuideBf16* wb, int p, float v) {
   const __nv_bfloat16 b = __float2bfloat16_rn(v);
@@ -760,18 +774,15 @@ __device__ __forceinline__ void write_bf16(GuideBf16* wb, int p, float v) {
 
 constexpr int kFoldBatch = 32;
 constexpr int kFoldThreads = 64;  // per CTA: the parameters spread over 87 SMs
-// fold the per-CTA partials in CTA order; lr > 0: one Adam step
+// parameter p: fold the per-CTA partials in CTA order; lr > 0: one Adam step
 // (Kingma & Ba 2015, beta1 = 0.9, beta2 = 0.999, eps = 1e-8) with the bias
-// corrections c1 = 1 / (1 - beta1^t), c2 = 1 / (1 - beta2^t)
-__global__ void k_guide_fold(const float* __restrict__ partials, int nparts, float* __restrict__ grad,
-                             float* __restrict__ w, float* __restrict__ m1, float* __restrict__ m2,
-                             GuideBf16* __restrict__ wb, float lr, float c1, float c2, float* __restrict__ loss_hist) {
-  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-  const int p = blockIdx.x * blockDim.x + threadIdx.x;
-  if (p >= kGPartial) return;
-  asm volatile("griddepcontrol.wait;" ::: "memory");
-  // in CTA order, kFoldBatch loads in flight (one after another, 64 partials
-  // cost 64 latencies of L2 in batches of 4)
+// corrections c1 = 1 / (1 - beta1^t), c2 = 1 / (1 - beta2^t).  kFoldBatch
+// partials are in flight (one after another in fours, 64 cost 16 latencies of
+// L2); all reads from L2: in the training kernel other CTAs wrote them
+__device__ __forceinline__ void fold_param(const float* __restrict__ partials, int nparts, int p,
+                                           float* __restrict__ grad, float* __restrict__ w, float* __restrict__ m1,
+                                           float* __restrict__ m2, GuideBf16* __restrict__ wb, float lr, float c1,
+                                           float c2, float* __restrict__ loss_hist) {
   float gsum = 0.0f;
   for (int b0 = 0; b0 < nparts; b0 += kFoldBatch) {
     float v[kFoldBatch];
@@ -794,6 +805,60 @@ __global__ void k_guide_fold(const float* __restrict__ partials, int nparts, flo
     const float wn = __ldcg(w + p) - lr * (a * c1) / (sqrtf(v * c2) + 1e-8f);
     w[p] = wn;
     write_bf16(wb, p, wn);
+  }
+}
+
+__global__ void k_guide_fold(const float* __restrict__ partials, int nparts, float* __restrict__ grad,
+                             float* __restrict__ w, float* __restrict__ m1, float* __restrict__ m2,
+                             GuideBf16* __restrict__ wb, float lr, float c1, float c2) {
+  const int p = blockIdx.x * blockDim.x + threadIdx.x;
+  if (p < kGPartial) fold_param(partials, nparts, p, grad, w, m1, m2, wb, lr, c1, c2, nullptr);
+}
+
+// all CTAs of a cooperative grid meet; a wait that runs out sets the error
+// word, and the CTA waits no more (`failed`)
+constexpr int kTrainWaitLimit = 1 << 21;
+__device__ __forceinline__ void train_barrier(unsigned* bar, unsigned target, int* err, bool& failed) {
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(bar) : "memory");
+    for (int i = 0; !failed; ++i) {
+      unsigned v;
+      asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(bar) : "memory");
+      if (v >= target) break;
+      if (i == kTrainWaitLimit) {
+        failed = true;
+        atomicExch(err, 1);
+      }
+    }
+  }
+  __syncthreads();
+}
+
+// `steps` training steps in one cooperative launch: gradient, barrier, fold and
+// Adam (the parameters spread over the CTAs), barrier.  Two launches per step
+// took 22.5 us (80k rows, batches of 4096), most of it latency; here a step
+// takes 11.6: the next step's samples are read while the barrier is waited for.  coef: (c1, c2) of each step; bar: 0 at launch.
+__global__ void __launch_bounds__(kGThreads) k_guide_train(GuideBf16* wb, float* w, GuideBatch B, long long step0,
+                                                           int steps, float* partials, float* grad, float* m1,
+                                                           float* m2, float lr, const float2* __restrict__ coef,
+                                                           float* loss_hist, unsigned* bar, int* err) {
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  TrainSmem& s = *reinterpret_cast<TrainSmem*>(smem_raw);
+  const int per = (kGPartial + gridDim.x - 1) / gridDim.x;
+  const int p0 = blockIdx.x * per, p1 = min(p0 + per, kGPartial);
+  bool failed = false;
+  unsigned target = 0;
+  float lab = load_samples(s, B, step0, blockIdx.x);
+  for (int k = 0; k < steps; ++k) {
+    grad_cta(s, wb, w, B, step0 + k, lab, partials + (size_t)blockIdx.x * kGPartial);
+    __syncthreads();  // the staged samples are used up
+    if (k + 1 < steps) lab = load_samples(s, B, step0 + k + 1, blockIdx.x);
+    train_barrier(bar, target += gridDim.x, err, failed);
+    const float2 c = coef[k];
+    for (int p = p0 + (int)threadIdx.x; p < p1; p += kGThreads)
+      fold_param(partials, gridDim.x, p, grad, w, m1, m2, wb, lr, c.x, c.y, loss_hist + k);
+    if (k + 1 < steps) train_barrier(bar, target += gridDim.x, err, failed);
   }
 }
 
@@ -844,7 +909,7 @@ int guide_check_error(pdhgc_guide* g, cudaStream_t st) {
   GK(cudaStreamSynchronize(st));
   if (e != 0) {
     GK(cudaMemsetAsync(g->err, 0, sizeof(int), st));
-    return set_error_detail(PDHGC_ERR_DEVICE, "a bounded tensor-core wait of the network ran out");
+    return set_error_detail(PDHGC_ERR_DEVICE, "a bounded wait of the network's kernels ran out");
   }
   return PDHGC_OK;
 }
@@ -853,8 +918,9 @@ int guide_step(pdhgc_guide* g, const __nv_bfloat16* feat, const uint8_t* labels,
                int batch, uint64_t seed, int64_t step, float adam_lr, cudaStream_t st) {
   const int nchunks = (batch + kChunk - 1) / kChunk;
   const int grid = nchunks < g->max_ctas ? nchunks : g->max_ctas;
-  k_guide_grad<<<grid, kGThreads, train_smem(), st>>>(g->wb, g->w, feat, labels, (long long)rows, idx, batch,
-                                                      (unsigned long long)seed, (long long)step, g->partials);
+  k_guide_grad<<<grid, kGThreads, train_smem(), st>>>(
+      g->wb, g->w, GuideBatch{feat, labels, (long long)rows, idx, batch, (unsigned long long)seed}, (long long)step,
+      g->partials);
   g->launches++;
   GKL();
   float c1 = 0.0f, c2 = 0.0f;
@@ -864,7 +930,7 @@ int guide_step(pdhgc_guide* g, const __nv_bfloat16* feat, const uint8_t* labels,
     c2 = (float)(1.0 / (1.0 - std::pow(0.999, (double)g->adam_t)));
   }
   k_guide_fold<<<(kGPartial + kFoldThreads - 1) / kFoldThreads, kFoldThreads, 0, st>>>(g->partials, grid, g->grad, g->w, g->m1, g->m2, g->wb,
-                                                        adam_lr, c1, c2, nullptr);
+                                                        adam_lr, c1, c2);
   g->launches++;
   GKL();
   return PDHGC_OK;
@@ -964,6 +1030,7 @@ void pdhgc_guide_destroy(pdhgc_guide* g) {
   cudaFree(g->wb);
   cudaFree(g->partials);
   cudaFree(g->idx);
+  cudaFree(g->train_buf);
   cudaFree(g->err);
   delete g;
 }
@@ -1091,49 +1158,45 @@ int pdhgc_guide_train(pdhgc_guide* g, const uint16_t* feat, const uint8_t* label
     return set_error_detail(PDHGC_ERR_INVALID_ARG, "NULL labels, batch <= 0, steps < 0 or lr <= 0");
   int rc = check_rows(feat, rows);
   if (rc != PDHGC_OK) return rc;
-  float* hist = nullptr;
-  if (losses && steps > 0) GK(cudaMallocAsync(&hist, sizeof(float) * (size_t)steps, g->stream));
-  for (int64_t s = 0; s < steps; ++s) {
-    // each kernel starts under the one before it (programmatic dependent
-    // launch; the first gradient kernel is ordered after the caller's work)
-    const int nchunks = (batch + kChunk - 1) / kChunk;
-    const int grid = nchunks < g->max_ctas ? nchunks : g->max_ctas;
+  if (!g->train_buf) {  // kept by the handle: (c1, c2) and the loss of each step of a launch, the barrier counter
+    GK(cudaMalloc(&g->train_buf, sizeof(float) * 3 * kTrainSteps + sizeof(unsigned)));
+    GK(cudaFuncSetAttribute(k_guide_train, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)train_smem()));
+  }
+  float2* const coef = reinterpret_cast<float2*>(g->train_buf);
+  float* const hist = g->train_buf + 2 * kTrainSteps;
+  unsigned* const bar = reinterpret_cast<unsigned*>(g->train_buf + 3 * kTrainSteps);
+  const int nchunks = (batch + kChunk - 1) / kChunk;
+  const int grid = nchunks < g->max_ctas ? nchunks : g->max_ctas;
+  const GuideBatch B{reinterpret_cast<const __nv_bfloat16*>(feat), labels, (long long)rows, nullptr, batch,
+                     (unsigned long long)seed};
+  std::vector<float2> c;
+  for (int64_t s0 = 0; s0 < steps; s0 += kTrainSteps) {
+    const int n = (int)(steps - s0 < kTrainSteps ? steps - s0 : kTrainSteps);
+    c.resize(n);
+    for (float2& q : c) {
+      g->adam_t++;
+      q.x = (float)(1.0 / (1.0 - std::pow(0.9, (double)g->adam_t)));
+      q.y = (float)(1.0 / (1.0 - std::pow(0.999, (double)g->adam_t)));
+    }
+    GK(cudaMemcpyAsync(coef, c.data(), sizeof(float2) * (size_t)n, cudaMemcpyHostToDevice, g->stream));
+    GK(cudaMemsetAsync(bar, 0, sizeof(unsigned), g->stream));
     cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    attr[0].id = cudaLaunchAttributeCooperative;
+    attr[0].val.cooperative = 1;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(grid);
     cfg.blockDim = dim3(kGThreads);
     cfg.dynamicSmemBytes = train_smem();
     cfg.stream = g->stream;
     cfg.attrs = attr;
-    cfg.numAttrs = s > 0 ? 1 : 0;
-    cudaError_t e = cudaLaunchKernelEx(&cfg, k_guide_grad, (const GuideBf16*)g->wb, (const float*)g->w,
-                                       reinterpret_cast<const __nv_bfloat16*>(feat), labels, (long long)rows,
-                                       (const int32_t*)nullptr, batch, (unsigned long long)seed, (long long)s,
-                                       g->partials);
-    g->adam_t++;
-    const float c1 = (float)(1.0 / (1.0 - std::pow(0.9, (double)g->adam_t)));
-    const float c2 = (float)(1.0 / (1.0 - std::pow(0.999, (double)g->adam_t)));
-    cfg.gridDim = dim3((kGPartial + kFoldThreads - 1) / kFoldThreads);
-    cfg.blockDim = dim3(kFoldThreads);
-    cfg.dynamicSmemBytes = 0;
     cfg.numAttrs = 1;
-    if (e == cudaSuccess)
-      e = cudaLaunchKernelEx(&cfg, k_guide_fold, (const float*)g->partials, grid, g->grad, g->w, g->m1, g->m2, g->wb,
-                             lr, c1, c2, hist ? hist + s : (float*)nullptr);
-    if (e == cudaSuccess) e = cudaGetLastError();
-    g->launches += 2;
-    if (e != cudaSuccess) {
-      if (hist) cudaFreeAsync(hist, g->stream);
-      return set_error_detail(PDHGC_ERR_CUDA, std::string("guide train launch: ") + cudaGetErrorString(e));
-    }
+    GK(cudaLaunchKernelEx(&cfg, k_guide_train, g->wb, g->w, B, (long long)s0, n, g->partials, g->grad, g->m1, g->m2, lr,
+                          (const float2*)coef, hist, bar, g->err));
+    g->launches++;
+    if (losses) GK(cudaMemcpyAsync(losses + s0, hist, sizeof(float) * (size_t)n, cudaMemcpyDeviceToHost, g->stream));
+    rc = guide_check_error(g, g->stream);  // also: c and hist are free again
+    if (rc != PDHGC_OK) return rc;
   }
-  if (hist) {
-    GK(cudaMemcpyAsync(losses, hist, sizeof(float) * (size_t)steps, cudaMemcpyDeviceToHost, g->stream));
-    GK(cudaFreeAsync(hist, g->stream));
-  }
-  GK(cudaStreamSynchronize(g->stream));
   return PDHGC_OK;
 }
 

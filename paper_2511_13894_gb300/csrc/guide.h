@@ -42,6 +42,7 @@ struct pdhgc_guide {
   float* partials = nullptr;  // per-CTA partial gradients
   int max_ctas = 0;
   int32_t* idx = nullptr;     // explicit minibatch indices (gradient check)
+  float* train_buf = nullptr;  // of the training kernel, allocated on first use
   int* err = nullptr;         // set by a kernel whose bounded wait ran out
   long long tc_wait_limit = 1ll << 24;  // polls of a tensor-core completion wait before it gives up
   int idx_cap = 0;
