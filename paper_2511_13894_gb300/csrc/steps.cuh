@@ -25,7 +25,7 @@
 //   FP64  200 x 500 random face 7.9 -> 3.4 (flow), 5000 x 17500 with bounds
 //         (averaged) 10.3 -> 5.1 (flow), 2000 x 8000 power law 13.8 -> 6.8 to 8.9
 //         (flow; it depends on where the entries lie in L2), 20k x 80k power law
-//         18.7 -> 12.9 (barrier)
+//         18.7 -> 12.7 (barrier)
 //   FP32  20k x 80k power law (averaged) 17.7 -> 12.4 (barrier)
 #pragma once
 #include "kernels.cuh"
@@ -289,6 +289,14 @@ __device__ __forceinline__ void step_pass(const Op& op, const StepLocal<typename
     step_fetch_hot(src, failed, err);
     __syncthreads();
   }
+  // the inputs of this warp's first joined rows: in barrier order they come from
+  // L2 (the barrier drops L1), which would follow the join
+  StepEpi ep{};
+  typename PF::Pre epre{};
+  if (!kFlow && warp < L.nepis) {
+    ep = L.epis[warp];
+    if (lane < ep.nrows) epre = PF::get(op, ep.row + lane);
+  }
   for (int t = L.t0; t < L.t1; ++t) {
     const StepTask k = L.tasks[t];
     const int np = k.np;
@@ -323,11 +331,12 @@ __device__ __forceinline__ void step_pass(const Op& op, const StepLocal<typename
   if (L.nepis > 0) {  // uniform over the CTA
     __syncthreads();
     for (int e = warp; e < L.nepis; e += kStepWarps) {
-      const StepEpi ep = L.epis[e];
+      if (kFlow || e != warp) {
+        ep = L.epis[e];
+        if (lane < ep.nrows) epre = PF::get(op, ep.row + lane);
+      }
       const int R = 32 >> ep.lg, r = lane & (R - 1);
       const bool has = r < ep.nrows;
-      typename PF::Pre pre{};
-      if (has && lane < R) pre = PF::get(op, ep.row + r);
       typename Op::Acc acc;
       acc.zero();
       if constexpr (std::is_same<VT, float>::value) {
@@ -339,7 +348,7 @@ __device__ __forceinline__ void step_pass(const Op& op, const StepLocal<typename
         for (int off = 16; off >= R; off >>= 1) acc.add(acc.shfl_xor(0xffffffffu, off));
       }
       if (has && lane < R) {
-        const typename Op::GT v = PF::epilogue_val(op, ep.row + r, acc, pre, part);
+        const typename Op::GT v = PF::epilogue_val(op, ep.row + r, acc, epre, part);
         if constexpr (kFlow) st_entry(dst + ep.row + r, v, seq);
       }
     }
