@@ -1281,6 +1281,31 @@ struct SpmvOp {
   }
 };
 
+// power iteration: out = (A_hat v) * inv[0] (inv null: 1); optional partial sum
+// of out^2
+template <bool kNorm>
+struct PiOp {
+  using Acc = SumD<1>;
+  static constexpr int NQ = kNorm ? 1 : 0;
+  static constexpr unsigned kMaxMask = 0;
+  const Scalars* S;
+  const double* v;
+  const double* inv;
+  double* out;
+  __device__ bool skip() const { return S->pi_zero != 0; }
+  __device__ double row_ctx(int) const { return 0.0; }
+  static constexpr int NG = 1;
+  using VT = double;
+  using GT = double;
+  __device__ const double* gsrc(int) const { return v; }
+  __device__ void accum(Acc& a, double, double val, const GV<double, 1>& g) const { a.v[0] = fma(val, g.v[0], a.v[0]); }
+  __device__ void epilogue(int r, const Acc& a, double* part) const {
+    const double x = inv ? a.v[0] * inv[0] : a.v[0];
+    out[r] = x;
+    if constexpr (kNorm) part[0] += x * x;
+  }
+};
+
 // Report on the ORIGINAL model for a given scaled point (x_hat, y_hat):
 // residual pieces plus the Section 2.1 / 4.2 slack metrics per row.
 struct ReportRowsOp {

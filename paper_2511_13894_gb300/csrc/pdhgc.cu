@@ -137,27 +137,23 @@ __global__ void k_norm2(const double* __restrict__ v, int n, double* out) {
   }
 }
 
-// power iteration: nw = ||w|| from partials; flag A_hat = 0
-__global__ void k_pi_norm(Scalars* S, const double* partials, int ntiles, double* nw_out) {
+// power iteration: 1 / ||w|| from partials; flag A_hat = 0
+__global__ void k_pi_norm(Scalars* S, const double* partials, int ntiles, double* inv_out) {
+  grid_dep_wait();
   __shared__ double s_tmp[32];
   if (S->pi_zero) return;
   const double s = block_fold(partials, ntiles, false, s_tmp);
   if (threadIdx.x == 0) {
     const double nw = sqrt(s);
-    nw_out[0] = nw;
+    inv_out[0] = 1.0 / nw;
     if (nw == 0.0) S->pi_zero = 1;
   }
-}
-
-__global__ void k_pi_scale(const Scalars* S, const double* w, const double* nw, double* v, int n) {
-  if (S->pi_zero) return;
-  const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i < n) v[i] = w[i] / nw[0];
 }
 
 // sigma_max, eta, initial primal weight
 __global__ void k_pi_final(Scalars* S, const double* partials, int ntiles, double eta_factor,
                            const double* nb2, const double* nc2) {
+  grid_dep_wait();
   __shared__ double s_tmp[32];
   double s = 0.0;
   if (!S->pi_zero) s = block_fold(partials, ntiles, false, s_tmp);
@@ -228,6 +224,7 @@ __global__ void k_to64(const Scalars* S, int n, int m, const float* __restrict__
                        const float2* __restrict__ sy, const double* __restrict__ lhat,
                        const double* __restrict__ uhat, double* __restrict__ x, double* __restrict__ y,
                        double* __restrict__ sum_x, double* __restrict__ sum_y) {
+  grid_dep_wait();
   if (S->done) return;
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i < n) {
@@ -309,6 +306,7 @@ __global__ void k_init_scalars(Scalars* S, PhaseInit pi, const double* cc2, unsi
 // steps i < P of the next chunk, t = steps since the anchor, and their
 // complements 1 / (t + i + 2) in FP32 (hs, FP32 bulk)
 __global__ void k_halpern_weights(const Scalars* S, double* hw, float* hs, int P) {
+  grid_dep_wait();
   if (S->done) return;
   const long long t = S->t;
   for (int i = threadIdx.x; i < P; i += blockDim.x) {
@@ -331,6 +329,7 @@ __global__ void k_h32_to64(const Scalars* S, int n, int m, const float* __restri
 // step kernel whose wait ran out (err) ends the phase.  seq: the step kernel's
 // counters (the next chunk's first step, its barrier)
 __global__ void k_pre_check(Scalars* S, unsigned* seq, const int* err) {
+  grid_dep_wait();
   if (threadIdx.x != 0 || S->done) return;
   seq[0] += (unsigned)S->check_period;
   seq[kStepBar] = 0u;
@@ -394,6 +393,7 @@ __device__ inline void group_fold(const Parts& part, int nq, unsigned max_mask, 
 // primal-weight update.  mode 0: initial restart point only.
 __global__ void k_decide(Scalars* S, const double* __restrict__ pA, int ntA, const double* __restrict__ pT,
                          int ntT, int mode, cudaGraphConditionalHandle h, int use_handle) {
+  grid_dep_wait();
   __shared__ double s_grp[kFoldGroups][8];
   __shared__ double q[22];
   if (S->done) {
@@ -424,6 +424,7 @@ __global__ void k_decide(Scalars* S, const double* __restrict__ pA, int ntA, con
 // Fold the 7 + 7 Halpern check quantities, then decide_halpern.
 __global__ void k_decide_h(Scalars* S, const double* __restrict__ pA, int ntA, const double* __restrict__ pT,
                            int ntT, int mode, cudaGraphConditionalHandle h, int use_handle) {
+  grid_dep_wait();
   __shared__ double s_grp[kFoldGroups][8];
   __shared__ double q[14];
   if (S->done) {
@@ -458,6 +459,7 @@ struct RingRec {
 // restart: jump to the candidate, new restart point, sums cleared.
 // restart_to 3 (Halpern loop): the iterate and the anchor become T(z).
 __global__ void k_restart_apply(const Scalars* S, int n, int m, DevIter w, Iter32 w32, RingRec rr, DevHalpern hz) {
+  grid_dep_wait();
   const int rt = S->restart_to;
   if (rt == 0 || S->done) return;
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
@@ -857,6 +859,24 @@ int launch_tiles(pdhgc_lp* lp, bool transposed, bool scaled, const Op& op, doubl
   return PDHGC_OK;
 }
 
+// a small kernel whose launch overlaps its predecessor's end: it waits
+// (grid_dep_wait) before it reads or writes anything
+template <class... Par, class... Arg>
+int launch_pdl(pdhgc_lp* lp, void (*kern)(Par...), int grid, int block, cudaStream_t st, Arg&&... arg) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(grid);
+  cfg.blockDim = dim3(block);
+  cfg.stream = st;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  CK(cudaLaunchKernelEx(&cfg, kern, std::forward<Arg>(arg)...));
+  lp->launches++;
+  return PDHGC_OK;
+}
+
 // the primal pass over A' as the chunked kernel (ChunkPlan): one CTA per SM,
 // the gathered vector staged in shared memory chunk by chunk
 template <class Op>
@@ -1179,15 +1199,17 @@ int setup_scaling(pdhgc_lp* lp, const pdhgc_params& p) {
     CKL();
     return PDHGC_OK;
   }
+  // u = A_hat v / ||v||, v = A_hat' u: the division is the row sums', so that v
+  // takes no pass of its own; the launches overlap their ramps (100k x 400k:
+  // 65 us per step with the fourth kernel and plain launches)
+  double* const inv = lp->scratch + 2;
   for (int k = 0; k < p.power_iters; ++k) {
-    RET(launch_tiles(lp, false, true, SpmvOp<false>{lp->S, lp->pi_v, lp->pi_u}, nullptr, st));
-    RET(launch_tiles(lp, true, true, SpmvOp<true>{lp->S, lp->pi_u, lp->pi_w}, lp->pT, st));
-    k_pi_norm<<<1, 1024, 0, st>>>(lp->S, lp->pT, lp->ntT, lp->scratch + 2);
-    k_pi_scale<<<grid_for(n), 256, 0, st>>>(lp->S, lp->pi_w, lp->scratch + 2, lp->pi_v, n);
-    lp->launches += 2;
-    CKL();
+    RET(launch_tiles(lp, false, true, PiOp<false>{lp->S, k ? lp->pi_w : lp->pi_v, k ? inv : nullptr, lp->pi_u},
+                     nullptr, st, true));
+    RET(launch_tiles(lp, true, true, SpmvOp<true>{lp->S, lp->pi_u, lp->pi_w}, lp->pT, st, true));
+    RET(launch_pdl(lp, k_pi_norm, 1, 1024, st, lp->S, (const double*)lp->pT, lp->ntT, inv));
   }
-  RET(launch_tiles(lp, false, true, SpmvOp<true>{lp->S, lp->pi_v, lp->pi_u}, lp->pA, st));
+  RET(launch_tiles(lp, false, true, PiOp<true>{lp->S, lp->pi_w, inv, lp->pi_u}, lp->pA, st, true));
   k_pi_final<<<1, 1024, 0, st>>>(lp->S, lp->pA, lp->ntA, p.eta_factor, lp->scratch + 0, lp->scratch + 1);
   lp->launches++;
   CKL();
@@ -1197,20 +1219,20 @@ int setup_scaling(pdhgc_lp* lp, const pdhgc_params& p) {
 // the KKT evaluation of the current and average points (two matrix passes)
 int launch_eval(pdhgc_lp* lp, const DevModel& md, cudaStream_t st, bool record_z) {
   const DevIter& w = lp->it;
-  RET(launch_tiles(lp, false, true, EvalRowsOp{lp->S, w.x, w.sum_x, w.y, w.sum_y, w.y_r, md}, lp->pA, st));
+  RET(launch_tiles(lp, false, true, EvalRowsOp{lp->S, w.x, w.sum_x, w.y, w.sum_y, w.y_r, md}, lp->pA, st, true));
   RET(launch_tiles(lp, true, true,
                    EvalColsOp{lp->S, w.y, w.sum_y, w.x, w.sum_x, w.x_r, md, record_z ? lp->z_cur : nullptr,
                               record_z ? lp->z_avg : nullptr},
-                   lp->pT, st));
+                   lp->pT, st, true));
   return PDHGC_OK;
 }
 
 // the Halpern check: T(z) and z - T(z) of the last step against the anchor
 int launch_eval_h(pdhgc_lp* lp, const DevModel& md, cudaStream_t st, bool record_z) {
   const DevIter& w = lp->it;
-  RET(launch_tiles(lp, false, true, EvalRowsH{lp->S, lp->hz, w.y_r, md}, lp->pA, st));
+  RET(launch_tiles(lp, false, true, EvalRowsH{lp->S, lp->hz, w.y_r, md}, lp->pA, st, true));
   RET(launch_tiles(lp, true, true, EvalColsH{lp->S, lp->hz, w.x_r, md, record_z ? lp->z_cur : nullptr}, lp->pT,
-                   st));
+                   st, true));
   return PDHGC_OK;
 }
 
@@ -1236,8 +1258,8 @@ DevH32 h32_of(const pdhgc_lp* lp) {
 // q = c_hat - A_hat' y_0 and r0 = b_hat - A_hat x_0 at the current anchor
 // (FP64 copies x_r, y_r); force = 0: only when the last decision restarted
 int launch_anchor(pdhgc_lp* lp, const DevModel& md, int force, cudaStream_t st) {
-  RET(launch_tiles(lp, true, true, AnchorColsOp{lp->S, force, lp->it.y_r, md.chat, lp->it32.q}, nullptr, st));
-  RET(launch_tiles(lp, false, true, AnchorRowsOp{lp->S, force, lp->it.x_r, md.bhat, lp->it32.r0}, nullptr, st));
+  RET(launch_tiles(lp, true, true, AnchorColsOp{lp->S, force, lp->it.y_r, md.chat, lp->it32.q}, nullptr, st, true));
+  RET(launch_tiles(lp, false, true, AnchorRowsOp{lp->S, force, lp->it.x_r, md.bhat, lp->it32.r0}, nullptr, st, true));
   return PDHGC_OK;
 }
 
@@ -1323,19 +1345,13 @@ int enqueue_body(pdhgc_lp* lp, const DevModel& md, const DevModel32& md32, const
     lp->launches++;
     rc = halpern ? launch_eval_h(lp, md, cs, ring) : launch_eval(lp, md, cs, ring);
   }
-  if (rc == PDHGC_OK) {
-    if (halpern)
-      k_decide_h<<<1, kFoldThreads, 0, cs>>>(lp->S, lp->pA, lp->ntA, lp->pT, lp->ntT, 1, handle, use_handle);
-    else
-      k_decide<<<1, kFoldThreads, 0, cs>>>(lp->S, lp->pA, lp->ntA, lp->pT, lp->ntT, 1, handle, use_handle);
-    k_restart_apply<<<gnm, 256, 0, cs>>>(lp->S, n, m, lp->it, w32, rr, hz);
-    lp->launches += 2;
-    if (halpern && fp32) rc = launch_anchor(lp, md, 0, cs);  // a restart moved the anchor
-    if (halpern && rc == PDHGC_OK) {
-      k_halpern_weights<<<1, 256, 0, cs>>>(lp->S, hz.hw, hz.hs, pi.check_period);
-      lp->launches++;
-    }
-  }
+  if (rc == PDHGC_OK)
+    rc = launch_pdl(lp, halpern ? k_decide_h : k_decide, 1, kFoldThreads, cs, lp->S, (const double*)lp->pA, lp->ntA,
+                    (const double*)lp->pT, lp->ntT, 1, handle, use_handle);
+  if (rc == PDHGC_OK) rc = launch_pdl(lp, k_restart_apply, gnm, 256, cs, (const Scalars*)lp->S, n, m, lp->it, w32, rr, hz);
+  if (rc == PDHGC_OK && halpern && fp32) rc = launch_anchor(lp, md, 0, cs);  // a restart moved the anchor
+  if (rc == PDHGC_OK && halpern)
+    rc = launch_pdl(lp, k_halpern_weights, 1, 256, cs, (const Scalars*)lp->S, hz.hw, hz.hs, pi.check_period);
   return rc;
 }
 
