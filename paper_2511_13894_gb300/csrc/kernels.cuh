@@ -466,44 +466,43 @@ __device__ __forceinline__ void row_dot_global(const Op& op, typename Op::Acc& a
   constexpr int NG = Op::NG;
   using VT = typename Op::VT;
   using GT = typename Op::GT;
-  int k = k0;
-  for (; k + (kBatch - 1) * step < k1; k += kBatch * step) {
-    VT v[kBatch];
-    int c[kBatch];
-    GV<GT, NG> g[kBatch];
+  // the next batch's matrix entries are requested while this batch's gathers
+  // are in flight: a long row is a chain of batches on one warp
+  VT v[kBatch];
+  int c[kBatch];
 #pragma unroll
-    for (int u = 0; u < kBatch; ++u) {
-      v[u] = ld_stream(val + k + u * step);
-      c[u] = ld_stream(col + k + u * step);
+  for (int u = 0; u < kBatch; ++u) {
+    c[u] = -1;
+    if (k0 + u * step < k1) {
+      v[u] = ld_stream(val + k0 + u * step);
+      c[u] = ld_stream(col + k0 + u * step);
     }
+  }
+  for (int k = k0; k < k1; k += kBatch * step) {
+    GV<GT, NG> g[kBatch];
 #pragma unroll
     for (int u = 0; u < kBatch; ++u)
+      if (c[u] >= 0)
 #pragma unroll
-      for (int i = 0; i < NG; ++i) g[u].v[i] = ld_gather(op.gsrc(i) + c[u]);
-#pragma unroll
-    for (int u = 0; u < kBatch; ++u) op.accum(acc, rc, v[u], g[u]);
-  }
-  // the ragged tail (fewer than kBatch entries left) as one predicated batch:
-  // its loads and gathers are in flight together, in the same summation order
-  if (k < k1) {
-    VT v[kBatch];
-    int c[kBatch];
-    GV<GT, NG> g[kBatch];
+        for (int i = 0; i < NG; ++i) g[u].v[i] = ld_gather(op.gsrc(i) + c[u]);
+    VT vn[kBatch];
+    int cn[kBatch];
 #pragma unroll
     for (int u = 0; u < kBatch; ++u) {
-      if (k + u * step < k1) {
-        v[u] = ld_stream(val + k + u * step);
-        c[u] = ld_stream(col + k + u * step);
+      cn[u] = -1;
+      if (k + (kBatch + u) * step < k1) {
+        vn[u] = ld_stream(val + k + (kBatch + u) * step);
+        cn[u] = ld_stream(col + k + (kBatch + u) * step);
       }
     }
 #pragma unroll
     for (int u = 0; u < kBatch; ++u)
-      if (k + u * step < k1)
+      if (c[u] >= 0) op.accum(acc, rc, v[u], g[u]);
 #pragma unroll
-        for (int i = 0; i < NG; ++i) g[u].v[i] = ld_gather(op.gsrc(i) + c[u]);
-#pragma unroll
-    for (int u = 0; u < kBatch; ++u)
-      if (k + u * step < k1) op.accum(acc, rc, v[u], g[u]);
+    for (int u = 0; u < kBatch; ++u) {
+      v[u] = vn[u];
+      c[u] = cn[u];
+    }
   }
 }
 
