@@ -366,22 +366,23 @@ __device__ inline void group_fold(const Parts& part, int nq, unsigned max_mask, 
     const int qi = r * kFoldGroups + g;
     const bool is_max = qi < nq && ((max_mask >> qi) & 1u);
     double v = 0.0;
+    int n = 0;
     if (qi < nq) {
       const double* p = nullptr;
-      int n = 0;
       part(qi, p, n);
       for (int k = t; k < n; k += 256) v = is_max ? fmax(v, p[k]) : v + p[k];
     }
-    for (int off = 16; off > 0; off >>= 1) {
-      const double o = __shfl_xor_sync(0xffffffffu, v, off);
-      v = is_max ? fmax(v, o) : v + o;
-    }
+    if (w * 32 < n)  // else all of the warp's values are 0: 160 FP64 warp operations less on the smallest LPs
+      for (int off = 16; off > 0; off >>= 1) {
+        const double o = __shfl_xor_sync(0xffffffffu, v, off);
+        v = is_max ? fmax(v, o) : v + o;
+      }
     __syncthreads();
     if (lane == 0) s_grp[g][w] = v;
     __syncthreads();
     if (qi < nq && t == 0) {
       double tot = s_grp[g][0];
-      for (int w2 = 1; w2 < 8; ++w2) tot = is_max ? fmax(tot, s_grp[g][w2]) : tot + s_grp[g][w2];
+      for (int w2 = 1; w2 < 8 && w2 * 32 < n; ++w2) tot = is_max ? fmax(tot, s_grp[g][w2]) : tot + s_grp[g][w2];
       q_out[qi] = tot;
     }
   }
