@@ -1000,7 +1000,9 @@ int fill_steps(pdhgc_lp* lp, const pdhgc_lp::Steps& sp, bool indices, cudaStream
 // above, copying the hot entries costs more than the barriers (5000 x 20000
 // power law, 0.16M: barrier 8.6, flow 9.5; 2000 x 8000, 0.06M: 8.1 and 6.8-8.9).
 constexpr int64_t kFlowMaxNnz = 65536;
-constexpr int kStepCtaNnz = 128;  // at least this many nonzeros per CTA: small LPs leave SMs to other handles
+// At least this much work per CTA (nonzeros, and two for each row and column):
+// small LPs leave SMs to other handles (200 x 500: 8, 16 and 152 CTAs within 2%)
+constexpr int kStepCtaWork = 128;
 
 template <class VT>
 int setup_steps_one(pdhgc_lp* lp, pdhgc_lp::Steps& sp, const Csr& A, const Csr& T, cudaStream_t st) {
@@ -1016,6 +1018,38 @@ int setup_steps_one(pdhgc_lp* lp, pdhgc_lp::Steps& sp, const Csr& A, const Csr& 
     sp.smem += sizeof(StepTask) * (size_t)P.max_tasks + sizeof(StepEpi) * (size_t)P.max_epis +
                2 * 8 * (size_t)P.max_part + (sizeof(VT) + sizeof(int)) * (size_t)P.max_slots;
   if (sp.smem > lp->step_smem_max) return PDHGC_OK;
+  // one upload and one allocation of device-filled arrays: a small LP's handle
+  // would spend longer on 28 copies than on its plans
+  std::vector<unsigned char> blob;
+  size_t room = 0;
+  auto at = [](size_t& end, size_t bytes) {  // the next 256-byte aligned place
+    const size_t off = (end + 255) & ~(size_t)255;
+    end = off + bytes;
+    return off;
+  };
+  auto pack = [&](const auto& v) {
+    size_t end = blob.size();
+    const size_t off = at(end, v.size() * sizeof(v[0]));
+    blob.resize(end);
+    if (!v.empty()) std::memcpy(blob.data() + off, v.data(), v.size() * sizeof(v[0]));
+    return off;
+  };
+  struct Offsets {
+    size_t tasks, epis, map, warp_ptr, epi_ptr, slot_ptr, slot0, col, val;
+  } off[2];
+  for (int t = 0; t < 2; ++t) {
+    const StepPlan& P = plan[t];
+    off[t] = {pack(P.tasks),    pack(P.epis),  pack(P.map), pack(P.warp_ptr), pack(P.epi_ptr),
+              pack(P.slot_ptr), pack(P.slot0), 0,           0};
+    off[t].col = at(room, sizeof(int) * (size_t)P.nslots);
+    off[t].val = at(room, sizeof(VT) * (size_t)P.nslots);
+  }
+  const size_t entry = lp->step_flow ? sizeof(typename StepEntry<VT>::type) : 0;
+  const size_t fx = at(room, entry * (size_t)lp->n), fy = at(room, entry * (size_t)lp->m);
+  unsigned char *d_plan, *d_room;
+  RET(lp->alloc(&d_plan, blob.size()));
+  RET(lp->alloc(&d_room, room));
+  CK(cudaMemcpyAsync(d_plan, blob.data(), blob.size(), cudaMemcpyHostToDevice, st));
   for (int t = 0; t < 2; ++t) {
     pdhgc_lp::StepSide& q = t ? sp.T : sp.A;
     const StepPlan& P = plan[t];
@@ -1024,32 +1058,20 @@ int setup_steps_one(pdhgc_lp* lp, pdhgc_lp::Steps& sp, const Csr& A, const Csr& 
     q.max_epis = P.max_epis;
     q.max_part = P.max_part;
     q.max_slots = P.max_slots;
-    auto up = [&](auto** dst, const auto& v) -> int {
-      RET(lp->alloc(dst, v.size()));
-      if (!v.empty()) CK(cudaMemcpyAsync(*dst, v.data(), v.size() * sizeof(v[0]), cudaMemcpyHostToDevice, st));
-      return PDHGC_OK;
-    };
-    RET(up(&q.tasks, P.tasks));
-    RET(up(&q.epis, P.epis));
-    RET(up(&q.map, P.map));
-    RET(up(&q.warp_ptr, P.warp_ptr));
-    RET(up(&q.epi_ptr, P.epi_ptr));
-    RET(up(&q.slot_ptr, P.slot_ptr));
-    RET(up(&q.slot0, P.slot0));
-    RET(lp->alloc(&q.col, (size_t)P.nslots));
-    VT* val;
-    RET(lp->alloc(&val, (size_t)P.nslots));
-    q.val = val;
+    q.tasks = reinterpret_cast<StepTask*>(d_plan + off[t].tasks);
+    q.epis = reinterpret_cast<StepEpi*>(d_plan + off[t].epis);
+    q.map = reinterpret_cast<StepSrcMap*>(d_plan + off[t].map);
+    q.warp_ptr = reinterpret_cast<int*>(d_plan + off[t].warp_ptr);
+    q.epi_ptr = reinterpret_cast<int*>(d_plan + off[t].epi_ptr);
+    q.slot_ptr = reinterpret_cast<int*>(d_plan + off[t].slot_ptr);
+    q.slot0 = reinterpret_cast<int*>(d_plan + off[t].slot0);
+    q.col = reinterpret_cast<int*>(d_room + off[t].col);
+    q.val = d_room + off[t].val;
   }
-  if (lp->step_flow) {
-    const size_t entry = sizeof(typename StepEntry<VT>::type);
-    unsigned char *fx, *fy;
-    RET(lp->alloc(&fx, entry * (size_t)lp->n));
-    RET(lp->alloc(&fy, entry * (size_t)lp->m));
-    CK(cudaMemsetAsync(fx, 0, entry * (size_t)lp->n, st));
-    CK(cudaMemsetAsync(fy, 0, entry * (size_t)lp->m, st));
-    sp.fx = fx;
-    sp.fy = fy;
+  if (lp->step_flow) {  // no entry is of a step yet
+    CK(cudaMemsetAsync(d_room + fx, 0, room - fx, st));
+    sp.fx = d_room + fx;
+    sp.fy = d_room + fy;
   }
   RET(fill_steps<VT>(lp, sp, true, st));
   CK(cudaStreamSynchronize(st));  // the plans go out of scope
@@ -1066,7 +1088,7 @@ int setup_steps(pdhgc_lp* lp, const Csr& A, const Csr& T, cudaStream_t st) {
   lp->step_smem_max = (size_t)smem - 1024;
   const double room = (double)sms * (double)lp->step_smem_max;
   if (!coop || 16.0 * (double)lp->nnz > room) return PDHGC_OK;
-  lp->step_ctas = (int)std::min<int64_t>(sms, std::max<int64_t>(1, lp->nnz / kStepCtaNnz));
+  lp->step_ctas = (int)std::min<int64_t>(sms, std::max<int64_t>(1, (lp->nnz + 2 * ((int64_t)lp->m + lp->n)) / kStepCtaWork));
   RET(lp->alloc(&lp->step_part, 2 * (size_t)lp->step_ctas));
   if (24.0 * (double)lp->nnz <= room) RET(setup_steps_one<double>(lp, lp->steps64, A, T, st));
   return setup_steps_one<float>(lp, lp->steps32, A, T, st);
