@@ -321,8 +321,8 @@ int pdhgc_set_launch_mode(pdhgc_lp* lp, int32_t mode);
  * status, iters and the phase fields are zero.  Work is enqueued on
  * `cuda_stream`, which the call synchronises.  The inputs are not
  * validated beyond NULL and size checks (use pdhgc_lp_create for that).
- * Scratch (n + 13 * 1024 + 16 doubles) is taken with cudaMallocAsync on
- * the stream and released before returning.  A'y is accumulated with
+ * Scratch (n + 15 * 608 + 16 doubles) is taken with cudaMallocAsync on
+ * the stream and freed on it before returning.  A'y is accumulated with
  * atomic adds, so results may differ from run to run in the last bits.
  * Errors: INVALID_ARG, OOM, CUDA.
  */
@@ -343,7 +343,7 @@ int pdhgc_kkt_eval(int32_t m, int32_t n, int64_t nnz, const int64_t* row_ptr, co
  *  - n must be <= 262,144 (1 << 18); a larger n returns PDHGC_ERR_TOO_LARGE
  *    without touching the device.
  *  - The scratch is a file-scope device array of 2,203,776 bytes ((1 << 18)
- *    + 13 * 1024 + 16 doubles) that every GPU which loads the library holds
+ *    + 15 * 608 + 16 doubles) that every GPU which loads the library holds
  *    until the process exits.  The call itself allocates nothing and calls
  *    no cudaMalloc, cudaFree or allocating library routine.
  *  - The first call on a device (the current device of the calling thread)
@@ -710,7 +710,10 @@ int pdhgc_probe_gather(int64_t n_vec, int64_t count, int32_t elem_bytes, int32_t
  * phase's model as plain launches on the handle's stream, each kernel
  * bracketed by CUDA events, and writes the mean duration in milliseconds of
  * one launch of the primal step (the A' pass, ms_out[0]) and of the dual
- * step (the A pass, ms_out[1]).  After a Halpern-loop phase the replayed
+ * step (the A pass, ms_out[1]).  Where the loop runs as one kernel per chunk
+ * (LPs whose matrix entries fit in the SMs' shared memory), one launch runs
+ * `iters` primal passes and another `iters` dual passes, and the means are per
+ * pass.  After a Halpern-loop phase the replayed
  * kernels are that loop's (a step inside a chunk, not a check step).  The
  * replayed iterations are real: they
  * advance the iterate state, which is left inconsistent with the phase's
