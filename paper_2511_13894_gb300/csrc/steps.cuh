@@ -62,7 +62,7 @@ struct StepFlow {
   const unsigned* seq;  // number of this launch's first step; grows from launch to launch
   unsigned* bar;        // barrier mode: arrivals, 0 at launch
   int* err;             // set when a bounded wait ran out
-  int hot_y, hot_x;            // leading entries of y / x_bar that every CTA copies to shared memory
+  int hot_y, hot_x;     // leading entries of y / x_bar that every CTA copies to shared memory
 };
 
 template <class T>
@@ -272,7 +272,7 @@ __device__ __forceinline__ void step_barrier(unsigned* bar, int* err, unsigned t
   __syncthreads();
 }
 
-// One matrix pass of this CTA.  s_part (the parts of CTA rows) alternates
+// One matrix pass of this CTA.  s_part (the parts of split rows) alternates
 // between two buffers from step to step: a warp may be a step ahead of another
 // that still adds parts, but not two (the barrier below).
 template <bool kFlow, class Op>
