@@ -711,9 +711,9 @@ int pdhgc_probe_gather(int64_t n_vec, int64_t count, int32_t elem_bytes, int32_t
  * bracketed by CUDA events, and writes the mean duration in milliseconds of
  * one launch of the primal step (the A' pass, ms_out[0]) and of the dual
  * step (the A pass, ms_out[1]).  Where the loop runs as one kernel per chunk
- * (LPs whose matrix entries fit in the SMs' shared memory), one launch runs
- * `iters` primal passes and another `iters` dual passes, and the means are per
- * pass.  After a Halpern-loop phase the replayed
+ * (LPs whose matrix entries fit in the SMs' shared memory), `iters` primal
+ * passes run first and then `iters` dual passes, up to 4096 in a launch, and
+ * the means are per pass.  After a Halpern-loop phase the replayed
  * kernels are that loop's (a step inside a chunk, not a check step).  The
  * replayed iterations are real: they
  * advance the iterate state, which is left inconsistent with the phase's

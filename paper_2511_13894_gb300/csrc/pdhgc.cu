@@ -71,6 +71,7 @@ struct DevReport {
   double p, d, cand;
 };
 
+constexpr int kMaxCheckPeriod = 4096;  // steps of a chunk, and Halpern weights kept for one
 constexpr int kStepBar = 32;  // the barrier counter's place in step_seq (a line of its own)
 
 // ---- small kernels ---------------------------------------------------------
@@ -1265,8 +1266,8 @@ int ensure_halpern(pdhgc_lp* lp) {
   RET(lp->alloc(&lp->hz.yp, (size_t)lp->m));
   RET(lp->alloc(&lp->hz.dx, (size_t)lp->n));
   RET(lp->alloc(&lp->hz.dy, (size_t)lp->m));
-  RET(lp->alloc(&lp->hz.hw, (size_t)4096));
-  RET(lp->alloc(&lp->hz.hs, (size_t)4096));
+  RET(lp->alloc(&lp->hz.hw, (size_t)kMaxCheckPeriod));
+  RET(lp->alloc(&lp->hz.hs, (size_t)kMaxCheckPeriod));
   lp->have_h = true;
   return PDHGC_OK;
 }
@@ -1556,7 +1557,7 @@ int fill_phase_report(pdhgc_lp* lp, pdhgc_report* r) {
 
 int check_params(const pdhgc_params* p) {
   if (!p) return PDHGC_ERR_INVALID_ARG;
-  if (p->max_iters < 1 || p->check_period < 1 || p->check_period > 4096 || p->ruiz_iters < 0 ||
+  if (p->max_iters < 1 || p->check_period < 1 || p->check_period > kMaxCheckPeriod || p->ruiz_iters < 0 ||
       p->ruiz_iters > 100 || p->power_iters < 1 || p->power_iters > 10000 || !(p->eta_factor > 0.0) ||
       !(p->eta_factor < 1.0) || !(p->time_limit_s > 0.0) || !(p->theta >= 0.0 && p->theta <= 1.0))
     return set_err(PDHGC_ERR_INVALID_ARG, "parameter out of range");
@@ -2888,15 +2889,20 @@ int pdhgc_profile_iteration(pdhgc_lp* lp, int32_t iters, double* ms_out) {
   const long long big = (long long)1 << 62;
   CK(cudaMemcpy(&lp->S->done, &zero, sizeof(int), cudaMemcpyHostToDevice));
   CK(cudaMemcpy(&lp->S->max_iters, &big, sizeof(long long), cudaMemcpyHostToDevice));
-  std::vector<cudaEvent_t> ev(3 * (size_t)iters + 1);
+  const bool steps = use_steps(lp, fp32, halpern);
+  std::vector<cudaEvent_t> ev(steps ? 4 : 3 * (size_t)iters);
   for (auto& e : ev) CK(cudaEventCreate(&e));
   int rc = PDHGC_OK;
-  if (use_steps(lp, fp32, halpern)) {
-    // the step kernel: all primal passes in one launch, then all dual passes
+  if (steps) {
+    // the step kernel: all primal passes, then all dual passes, in launches of
+    // at most kMaxCheckPeriod (a solve's longest; the barrier counts in 32 bits)
     for (int pass = 0; pass < 2 && rc == PDHGC_OK; ++pass) {
-      CK(cudaMemsetAsync(lp->step_seq + kStepBar, 0, sizeof(unsigned), st));
       CK(cudaEventRecord(ev[2 * pass], st));
-      rc = enqueue_steps(lp, md, md32, halpern, fp32, lp->params.reflection, iters, 1, 1 << pass, st);
+      for (int left = iters; left > 0 && rc == PDHGC_OK; left -= kMaxCheckPeriod) {
+        CK(cudaMemsetAsync(lp->step_seq + kStepBar, 0, sizeof(unsigned), st));
+        rc = enqueue_steps(lp, md, md32, halpern, fp32, lp->params.reflection, std::min(left, kMaxCheckPeriod), 1,
+                           1 << pass, st);
+      }
       CK(cudaEventRecord(ev[2 * pass + 1], st));
     }
     CK(cudaMemsetAsync(lp->step_seq + kStepBar, 0, sizeof(unsigned), st));

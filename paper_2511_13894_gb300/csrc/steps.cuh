@@ -422,8 +422,8 @@ __global__ void __launch_bounds__(kStepThreads, 1)
   unsigned target = 0;
   __syncthreads();
   for (int i = 0; i < n_it; ++i) {
-    opT.it = i;
-    opA.it = i;
+    opT.it = both ? i : 0;  // a timed pass replays a step inside a chunk: the Halpern weights end with the chunk
+    opA.it = opT.it;
     const unsigned seq = both ? seq0 + (unsigned)i : 0u;
     if (which & 1) {
       if (!kFlow && target) step_barrier(flow.bar, flow.err, target, failed);
