@@ -310,6 +310,16 @@ int pdhgc_set_primal_layout(pdhgc_lp* lp, int32_t chunked);
 int pdhgc_set_launch_mode(pdhgc_lp* lp, int32_t mode);
 
 /*
+ * pdhgc_set_wait_limit — polls each wait of a kernel whose CTAs wait for each
+ * other (the step kernel and the power iteration of LPs whose matrix entries
+ * fit in the SMs' shared memory) makes before it gives up: 0 (give up at once)
+ * to 2^21 (the default, about a second; larger values count as this one).  A
+ * wait that gives up makes the call return DEVICE, its results are void, and
+ * the handle stays usable.  For failure-path tests.  Errors: INVALID_ARG.
+ */
+int pdhgc_set_wait_limit(pdhgc_lp* lp, int64_t polls);
+
+/*
  * pdhgc_kkt_eval — the Section 2 residuals, objectives and relative ratios,
  * and the Section 2.1 / 4.2 metrics, of a caller-supplied point (x, y) on an
  * LP given as device arrays, without creating a handle.  The LP arguments
@@ -677,9 +687,10 @@ int64_t pdhgc_guide_kernel_launches(const pdhgc_guide* g);
  * back).  set_state restores into a handle created from the same LP: it
  * recomputes the scaling and step size (deterministic) and returns INVALID_ARG
  * when the shape, the format or the recomputed scaling factors differ from the
- * saved ones.  Afterwards get_solution, kkt_report, corner_phase and the
- * guidance calls behave as on the original handle.  The state is not portable
- * across builds that change the scaling arithmetic.
+ * saved ones, DEVICE when a wait of the recomputation ran out.  Afterwards
+ * get_solution, kkt_report, corner_phase and the guidance calls behave as on
+ * the original handle.  The state is not portable across builds that change
+ * the scaling arithmetic.
  */
 int pdhgc_get_state(pdhgc_lp* lp, void* buf, size_t* bytes);
 int pdhgc_set_state(pdhgc_lp* lp, const void* buf, size_t bytes);
@@ -718,7 +729,7 @@ int pdhgc_probe_gather(int64_t n_vec, int64_t count, int32_t elem_bytes, int32_t
  * replayed iterations are real: they
  * advance the iterate state, which is left inconsistent with the phase's
  * report (x1/y1 and the corner result are not touched).  For profiling.
- * Errors: NO_PHASE1, INVALID_ARG (iters < 1 or ms_out NULL).
+ * Errors: NO_PHASE1, INVALID_ARG (iters < 1 or ms_out NULL), CUDA, DEVICE.
  */
 int pdhgc_profile_iteration(pdhgc_lp* lp, int32_t iters, double* ms_out);
 

@@ -800,6 +800,7 @@ struct pdhgc_lp {
   double *pi_v = nullptr, *pi_w = nullptr, *pi_u = nullptr, *tmp_n = nullptr, *tmp_m = nullptr;
   double *pA = nullptr, *pT = nullptr, *scratch = nullptr;
   int* err = nullptr;  // device error word set by a kernel whose bounded wait ran out
+  int wait_limit = kStepWaitLimit;  // pdhgc_set_wait_limit
   Scalars* S = nullptr;
   DevReport* rep = nullptr;
   double b_norm = 0.0, c_norm = 0.0;
@@ -937,7 +938,8 @@ StepMat<VT> steps_side(const pdhgc_lp::StepSide& q) {
 }
 
 StepFlow steps_flow(const pdhgc_lp* lp, const pdhgc_lp::Steps& sp) {
-  return StepFlow{sp.fy, sp.fx, lp->step_seq, lp->step_seq + kStepBar, lp->err, sp.hot_y, sp.hot_x};
+  return StepFlow{sp.fy, sp.fx, lp->step_seq, lp->step_seq + kStepBar, lp->err, lp->wait_limit,
+                  sp.hot_y, sp.hot_x};
 }
 
 // a cooperative launch of the step CTAs; the limit on dynamic shared memory is
@@ -1437,6 +1439,17 @@ int launch_loop(pdhgc_lp* lp, const DevModel& md, const DevModel32& md32, const 
   return PDHGC_OK;
 }
 
+// DEVICE when a kernel launched since the last call gave up a wait; read at the
+// end of every call that launches such kernels, so that none reports another's
+int take_error(pdhgc_lp* lp) {
+  int derr = 0;
+  CK(cudaMemcpyAsync(&derr, lp->err, sizeof(int), cudaMemcpyDeviceToHost, lp->stream));
+  CK(cudaStreamSynchronize(lp->stream));
+  if (derr == 0) return PDHGC_OK;
+  CK(cudaMemsetAsync(lp->err, 0, sizeof(int), lp->stream));
+  return set_err(PDHGC_ERR_DEVICE, "a bounded device wait ran out (error word " + std::to_string(derr) + ")");
+}
+
 // Runs one phase: init, the device-driven loop graph, finalize.
 int run_phase(pdhgc_lp* lp, const DevModel& md, const DevModel32& md32, const PhaseInit& pi,
               const double* x_start, const double* cc2, double* xo, double* yo, const double* x_fallback,
@@ -1497,13 +1510,7 @@ int run_phase(pdhgc_lp* lp, const DevModel& md, const DevModel32& md32, const Ph
     lp->launches++;
   }
   CKL();
-  CK(cudaStreamSynchronize(st));
-  int derr = 0;
-  CK(cudaMemcpy(&derr, lp->err, sizeof(int), cudaMemcpyDeviceToHost));
-  if (derr != 0) CK(cudaMemset(lp->err, 0, sizeof(int)));  // reported once
-  if (derr != 0) return set_err(PDHGC_ERR_DEVICE, "a bounded device wait ran out (error word " +
-                                                      std::to_string(derr) + ")");
-  return PDHGC_OK;
+  return take_error(lp);
 }
 
 int run_report(pdhgc_lp* lp, const double* x, const double* y, pdhgc_report* out) {
@@ -2607,6 +2614,7 @@ int pdhgc_set_state(pdhgc_lp* lp, const void* buf, size_t bytes) {
     RET(ensure_fp32(lp));
     RET(convert_fp32(lp, st));
   }
+  RET(take_error(lp));
   std::vector<double> Dr(m), Dc(n);
   CK(cudaMemcpyAsync(Dr.data(), lp->Dr, 8 * (size_t)m, cudaMemcpyDeviceToHost, st));
   CK(cudaMemcpyAsync(Dc.data(), lp->Dc, 8 * (size_t)n, cudaMemcpyDeviceToHost, st));
@@ -2857,6 +2865,12 @@ int pdhgc_set_launch_mode(pdhgc_lp* lp, int32_t mode) {
   return PDHGC_OK;
 }
 
+int pdhgc_set_wait_limit(pdhgc_lp* lp, int64_t polls) {
+  if (!lp || polls < 0) return set_err(PDHGC_ERR_INVALID_ARG, "lp is NULL or polls < 0");
+  lp->wait_limit = (int)std::min<int64_t>(polls, kStepWaitLimit);
+  return PDHGC_OK;
+}
+
 int pdhgc_get_layout(const pdhgc_lp* lp, int64_t* out) {
   if (!lp || !out) return set_err(PDHGC_ERR_INVALID_ARG, "bad argument");
   const pdhgc_lp::Mat* mats[2] = {&lp->A, &lp->T};
@@ -2915,7 +2929,8 @@ int pdhgc_profile_iteration(pdhgc_lp* lp, int32_t iters, double* ms_out) {
     for (auto& e : ev) cudaEventDestroy(e);
     CK(cudaMemcpy(&lp->S->done, &saved_done, sizeof(int), cudaMemcpyHostToDevice));
     CK(cudaMemcpy(&lp->S->max_iters, &saved_max, sizeof(long long), cudaMemcpyHostToDevice));
-    return rc;
+    const int waited = take_error(lp);
+    return rc != PDHGC_OK ? rc : waited;
   }
   for (int i = 0; i < iters && rc == PDHGC_OK; ++i) {
     CK(cudaEventRecord(ev[3 * i], st));

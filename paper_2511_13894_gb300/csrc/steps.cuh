@@ -62,6 +62,7 @@ struct StepFlow {
   const unsigned* seq;  // number of this launch's first step; grows from launch to launch
   unsigned* bar;        // barrier mode: arrivals, 0 at launch
   int* err;             // set when a bounded wait ran out
+  int limit;            // polls of one wait before that
   int hot_y, hot_x;     // leading entries of y / x_bar that every CTA copies to shared memory
 };
 
@@ -113,7 +114,7 @@ __device__ __forceinline__ float ld_iter(const float* p) {
 // registers) are what 128 registers hold without spilling.
 template <bool kFlow, class VT>
 constexpr int kStepPairs = std::is_same<VT, float>::value ? (kFlow ? 4 : 8) : 2;
-constexpr int kStepWaitLimit = 1 << 21;        // polls of one gather (about a second)
+constexpr int kStepWaitLimit = 1 << 21;        // polls of one wait (about a second); a handle can set fewer
 
 __device__ __forceinline__ void ld_entry(const ulonglong2* p, double& v, unsigned& seq) {
   unsigned long long a, b;
@@ -174,7 +175,7 @@ struct StepSrc {
 
 // copies the hot values of step `want` into shared memory
 template <class GT>
-__device__ __forceinline__ void step_fetch_hot(const StepSrc<GT>& src, bool& failed, int* err) {
+__device__ __forceinline__ void step_fetch_hot(const StepSrc<GT>& src, bool& failed, int* err, int limit) {
   for (int j = threadIdx.x; j < src.n_hot; j += kStepThreads) {
     GT v;
     unsigned q;
@@ -182,7 +183,7 @@ __device__ __forceinline__ void step_fetch_hot(const StepSrc<GT>& src, bool& fai
       ld_entry(src.entries + j, v, q);
       if ((int)(q - src.want) >= 0 || failed) break;  // newer: all rows that read entry j are done
       if (i > 256) __nanosleep(100);
-      if (i == kStepWaitLimit) {
+      if (i >= limit) {
         failed = true;
         atomicExch(err, 2);
       }
@@ -195,7 +196,8 @@ __device__ __forceinline__ void step_fetch_hot(const StepSrc<GT>& src, bool& fai
 template <bool kFlow, int PB, class Op>
 __device__ __forceinline__ void step_consume(const Op& op, typename Op::Acc& acc,
                                              const StepHead<typename Op::VT, PB>& h,
-                                             const StepSrc<typename Op::GT>& src, bool& failed, int* err) {
+                                             const StepSrc<typename Op::GT>& src, bool& failed, int* err,
+                                             int limit) {
   using GT = typename Op::GT;
   constexpr int B = 2 * PB;
   GV<GT, 1> g[B];
@@ -226,7 +228,7 @@ __device__ __forceinline__ void step_consume(const Op& op, typename Op::Acc& acc
       stale = false;
 #pragma unroll
       for (int u = 0; u < B; ++u) stale |= q[u] != src.want;
-      if (i == kStepWaitLimit) {  // uniform in the warp: it waits no more in this launch
+      if (i >= limit) {  // uniform in the warp: it waits no more in this launch
         failed = true;
         if ((threadIdx.x & 31) == 0) atomicExch(err, 2);
       }
@@ -255,17 +257,17 @@ struct StepLocal {
 
 // the grid's barrier (barrier mode): `target` arrivals in all.  A wait that
 // runs out sets the error word, and the CTA waits no more in this launch
-__device__ __forceinline__ void step_barrier(unsigned* bar, int* err, unsigned target, bool& failed) {
+__device__ __forceinline__ void step_barrier(const StepFlow& flow, unsigned target, bool& failed) {
   __syncthreads();
   if (threadIdx.x == 0) {
-    asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(bar) : "memory");
+    asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(flow.bar) : "memory");
     for (int i = 0; !failed; ++i) {
       unsigned v;
-      asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(bar) : "memory");
+      asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(flow.bar) : "memory");
       if (v >= target) break;
-      if (i == kStepWaitLimit) {
+      if (i >= flow.limit) {
         failed = true;
-        atomicExch(err, 2);
+        atomicExch(flow.err, 2);
       }
     }
   }
@@ -279,14 +281,14 @@ template <bool kFlow, class Op>
 __device__ __forceinline__ void step_pass(const Op& op, const StepLocal<typename Op::VT>& L,
                                           typename Op::Acc* __restrict__ s_part, const StepSrc<typename Op::GT>& src,
                                           typename StepEntry<typename Op::GT>::type* __restrict__ dst, unsigned seq,
-                                          bool& failed, int* err, double* part) {
+                                          bool& failed, int* err, int limit, double* part) {
   using VT = typename Op::VT;
   using V2 = typename Vec2<VT>::type;
   using PF = Prefetcher<Op>;
   constexpr int PB = kStepPairs<kFlow, VT>;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   if (kFlow && src.wait && src.n_hot > 0) {  // uniform over the grid
-    step_fetch_hot(src, failed, err);
+    step_fetch_hot(src, failed, err, limit);
     __syncthreads();
   }
   // the inputs of this warp's first joined rows: in barrier order they come from
@@ -311,7 +313,7 @@ __device__ __forceinline__ void step_pass(const Op& op, const StepLocal<typename
     if (lead) pre = PF::get(op, k.row + lane);
     for (int p = 0; p < np; p += PB) {
       step_load<VT, PB>(head, vp, cp, p, np);
-      step_consume<kFlow, PB>(op, acc, head, src, failed, err);
+      step_consume<kFlow, PB>(op, acc, head, src, failed, err, limit);
     }
     // lanes 0 .. R - 1 hold the rows' parts 0, the next R their parts 1 ...
     const int lg = k.flags & kStepLgMask, R = 32 >> lg;
@@ -426,16 +428,16 @@ __global__ void __launch_bounds__(kStepThreads, 1)
     opA.it = opT.it;
     const unsigned seq = both ? seq0 + (unsigned)i : 0u;
     if (which & 1) {
-      if (!kFlow && target) step_barrier(flow.bar, flow.err, target, failed);
+      if (!kFlow && target) step_barrier(flow, target, failed);
       target += gridDim.x;
       step_pass<kFlow>(opT, LT, part_t + (i & 1) * T.max_part, StepSrc<GT>{fy, seq - 1, both && i > 0, s_hy, flow.hot_y},
-                       fx, seq, failed, flow.err, nullptr);
+                       fx, seq, failed, flow.err, flow.limit, nullptr);
     }
     if (which & 2) {
-      if (!kFlow && target) step_barrier(flow.bar, flow.err, target, failed);
+      if (!kFlow && target) step_barrier(flow, target, failed);
       target += gridDim.x;
       step_pass<kFlow>(opA, LA, part_a + (i & 1) * A.max_part, StepSrc<GT>{fx, seq, both, s_hx, flow.hot_x}, fy, seq,
-                       failed, flow.err, nullptr);
+                       failed, flow.err, flow.limit, nullptr);
     }
   }
 }
@@ -499,16 +501,16 @@ __global__ void __launch_bounds__(kStepThreads, 1)
   ulonglong2* const none = nullptr;
   for (int k = 0; k <= iters; ++k) {
     double sq = 0.0;
-    step_pass<false>(PowerOp{k == 0 ? v : w, u, scale}, LA, part_a, plain, none, 0u, failed, flow.err, &sq);
+    step_pass<false>(PowerOp{k == 0 ? v : w, u, scale}, LA, part_a, plain, none, 0u, failed, flow.err, flow.limit, &sq);
     if (k == iters) {
       block_sum(sq, partials);
       return;
     }
-    step_barrier(flow.bar, flow.err, target += gridDim.x, failed);
+    step_barrier(flow, target += gridDim.x, failed);
     sq = 0.0;
-    step_pass<false>(PowerOp{u, w, 1.0}, LT, part_t, plain, none, 0u, failed, flow.err, &sq);
+    step_pass<false>(PowerOp{u, w, 1.0}, LT, part_t, plain, none, 0u, failed, flow.err, flow.limit, &sq);
     block_sum(sq, norm_part);
-    step_barrier(flow.bar, flow.err, target += gridDim.x, failed);
+    step_barrier(flow, target += gridDim.x, failed);
     if (warp == 0) {
       double x = 0.0;
       for (int b = lane; b < (int)gridDim.x; b += 32) x += __ldcg(norm_part + b);

@@ -112,6 +112,7 @@ _sig = {
     "pdhgc_get_layout": (C.c_int, [_vp, _vp]),
     "pdhgc_set_primal_layout": (C.c_int, [_vp, C.c_int32]),
     "pdhgc_set_launch_mode": (C.c_int, [_vp, C.c_int32]),
+    "pdhgc_set_wait_limit": (C.c_int, [_vp, C.c_int64]),
     "pdhgc_uniform": (C.c_int, [C.c_uint64, C.c_int64, C.c_double, _vp, _vp]),
     "pdhgc_kkt_eval": (C.c_int, [C.c_int32, C.c_int32, C.c_int64, _vp, _vp, _vp, _vp, _vp, _vp, _vp, _vp, _vp,
                                  _vp, C.POINTER(Report), _vp]),
@@ -287,6 +288,10 @@ class LP:
         """pdhgc_set_launch_mode: LAUNCH_GRAPH (default, one conditional graph
         per phase) or LAUNCH_STREAM (plain launches, one body at a time)."""
         _check(lib.pdhgc_set_launch_mode(self._h, int(mode)), "pdhgc_set_launch_mode")
+
+    def set_wait_limit(self, polls: int):
+        """pdhgc_set_wait_limit (failure-path tests)."""
+        _check(lib.pdhgc_set_wait_limit(self._h, int(polls)), "pdhgc_set_wait_limit")
 
     def set_primal_layout(self, chunked: bool):
         """pdhgc_set_primal_layout: 0 gathers from global memory (default), 1 stages y in shared memory."""

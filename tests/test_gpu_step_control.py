@@ -1,9 +1,10 @@
-"""The persistent step kernel outside a plain solve: replayed passes (needs a GB300)."""
+"""The persistent step kernel outside a plain solve: replayed passes, waits that run out (needs a GB300)."""
 import numpy as np
 import pytest
 
 import lpgen
 from tests.test_gpu_parity import ITER_TOL, rel_err
+from tests.test_gpu_steps import CASES
 
 pytestmark = pytest.mark.gpu
 
@@ -55,4 +56,53 @@ def test_replayed_passes_are_steps_inside_a_chunk(iters, precision):
     again = g.get_iterates()
     for k in ("x", "y", "x_avg", "y_avg"):
         assert np.array_equal(again[k], it[k]), k
+    g.close()
+
+
+def _device_error(f, *a, **kw):
+    with pytest.raises(P.PdhgcError) as e:
+        f(*a, **kw)
+    assert e.value.code == -10
+
+
+def _results(g):
+    return [*g.get_solution(P.PHASE1), *g.get_solution(P.CORNER), *(g.get_iterates()[k] for k in ("x", "y"))]
+
+
+# flow order, flow order with hot copies, barrier order; a few tens of CTAs or more each: two that run in step may
+# never find a value missing
+ORDERS = {"flow": lambda: lpgen.small_face_lp(2), "hot": CASES["hot_lengths"], "barrier": CASES["barrier_order"]}
+
+
+@pytest.mark.parametrize("precision", ["fp64", "fp32"])
+@pytest.mark.parametrize("name", list(ORDERS))
+def test_a_wait_that_runs_out_is_reported_by_its_own_call(name, precision):
+    """Failure detection without a fault: waits that give up at once make the solve, the corner phase, a restored
+    state and (in barrier order) the replayed passes return DEVICE; the next call gives the handle's usual bits."""
+    lp = ORDERS[name]()
+    kw = dict(max_iters=256, eps_rel=-1.0, algorithm=P.HALPERN,
+              precision=P.FP64 if precision == "fp64" else P.FP32_BULK)
+    ckw = dict(obj_seed=3, eps_rel=1e30, min_iters=128)
+    g = P.lp_from_dict(lp)
+    g.solve(**kw)
+    state = g.get_state()
+    g.corner_phase(**ckw)
+    want = _results(g)
+    if name == "barrier":
+        g.set_wait_limit(0)
+        _device_error(g.profile_iteration, 8)
+        g.set_wait_limit(1 << 21)
+        assert min(g.profile_iteration(8)) > 0
+    g.set_wait_limit(0)  # the power iteration's waits
+    _device_error(g.solve, **kw)
+    _device_error(g.set_state, state)
+    g.set_wait_limit(1 << 21)
+    g.set_state(state)
+    g.solve(**kw)
+    g.set_wait_limit(0)
+    _device_error(g.corner_phase, **ckw)
+    g.set_wait_limit(1 << 21)
+    g.corner_phase(**ckw)
+    for a, b in zip(_results(g), want):
+        assert np.array_equal(a, b)
     g.close()
