@@ -602,7 +602,7 @@ int pdhgc_guide_load(pdhgc_guide* g, const char* path);
 /*
  * pdhgc_guide_infer — probabilities p[r] for `rows` feature rows; feat and p
  * are DEVICE pointers (feat: rows x 32 BF16, 16-byte aligned; p: rows FP32).
- * Errors: INVALID_ARG (NULL, rows < 1, misaligned), CUDA.
+ * Errors: INVALID_ARG (NULL, rows < 1, misaligned), CUDA, DEVICE.
  */
 int pdhgc_guide_infer(pdhgc_guide* g, const uint16_t* feat, int64_t rows, float* p);
 
@@ -621,7 +621,9 @@ int pdhgc_guide_grad(pdhgc_guide* g, const uint16_t* feat, const uint8_t* labels
  * of `batch` rows drawn with replacement: row SplitMix64(seed, step * batch
  * + s) mod rows for s < batch.  feat and labels are DEVICE arrays as above;
  * losses (host, `steps` floats, may be NULL) receives each step's minibatch
- * loss.  Errors: INVALID_ARG, CUDA, OOM.
+ * loss.  Errors: INVALID_ARG, CUDA, OOM, DEVICE (a wait between the GPU's SMs
+ * ran out: the weights and Adam's moments are then undefined until
+ * pdhgc_guide_set_weights or _load sets them).
  */
 int pdhgc_guide_train(pdhgc_guide* g, const uint16_t* feat, const uint8_t* labels, int64_t rows, int32_t batch,
                       int64_t steps, float lr, uint64_t seed, float* losses);
@@ -668,7 +670,8 @@ int pdhgc_corner_phase_guided(pdhgc_lp* lp, const pdhgc_corner_params* params, c
 /*
  * pdhgc_guide_set_wait_limit — polls each tensor-core completion wait of the
  * inference kernel makes before it gives up (default 2^24; 0: give up at
- * once).  A wait that gives up makes the call return DEVICE; the kernel
+ * once), and each grid wait of the training kernel (the same number, 2^21 at
+ * most).  A wait that gives up makes the call return DEVICE; the kernel
  * still lets the pending product land (full limit) and frees its tensor
  * memory, so the context stays usable.  For failure-path tests.
  */

@@ -21,6 +21,7 @@
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
 
+#include <algorithm>
 #include <cmath>
 #include <cstdio>
 #include <cstring>
@@ -818,8 +819,8 @@ __global__ void k_guide_fold(const float* __restrict__ partials, int nparts, flo
 
 // all CTAs of a cooperative grid meet; a wait that runs out sets the error
 // word, and the CTA waits no more (`failed`)
-constexpr int kTrainWaitLimit = 1 << 21;
-__device__ __forceinline__ void train_barrier(unsigned* bar, unsigned target, int* err, bool& failed) {
+constexpr int kTrainWaitLimit = 1 << 21;  // polls (about a second); pdhgc_guide_set_wait_limit can set fewer
+__device__ __forceinline__ void train_barrier(unsigned* bar, unsigned target, int* err, int limit, bool& failed) {
   __syncthreads();
   if (threadIdx.x == 0) {
     asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(bar) : "memory");
@@ -827,7 +828,7 @@ __device__ __forceinline__ void train_barrier(unsigned* bar, unsigned target, in
       unsigned v;
       asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(bar) : "memory");
       if (v >= target) break;
-      if (i == kTrainWaitLimit) {
+      if (i >= limit) {
         failed = true;
         *reinterpret_cast<volatile int*>(err) = 1;
       }
@@ -843,7 +844,7 @@ __device__ __forceinline__ void train_barrier(unsigned* bar, unsigned target, in
 __global__ void __launch_bounds__(kGThreads) k_guide_train(GuideBf16* wb, float* w, GuideBatch B, long long step0,
                                                            int steps, float* partials, float* grad, float* m1,
                                                            float* m2, float lr, const float2* __restrict__ coef,
-                                                           float* loss_hist, unsigned* bar, int* err) {
+                                                           float* loss_hist, unsigned* bar, int* err, int limit) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   TrainSmem& s = *reinterpret_cast<TrainSmem*>(smem_raw);
   const int per = (kGPartial + gridDim.x - 1) / gridDim.x;
@@ -855,11 +856,11 @@ __global__ void __launch_bounds__(kGThreads) k_guide_train(GuideBf16* wb, float*
     grad_cta(s, wb, w, B, step0 + k, lab, partials + (size_t)blockIdx.x * kGPartial);
     __syncthreads();  // the staged samples are used up
     if (k + 1 < steps) lab = load_samples(s, B, step0 + k + 1, blockIdx.x);
-    train_barrier(bar, target += gridDim.x, err, failed);
+    train_barrier(bar, target += gridDim.x, err, limit, failed);
     const float2 c = coef[k];
     for (int p = p0 + (int)threadIdx.x; p < p1; p += kGThreads)
       fold_param(partials, gridDim.x, p, grad, w, m1, m2, wb, lr, c.x, c.y, loss_hist + k);
-    if (k + 1 < steps) train_barrier(bar, target += gridDim.x, err, failed);
+    if (k + 1 < steps) train_barrier(bar, target += gridDim.x, err, limit, failed);
   }
 }
 
@@ -897,7 +898,7 @@ int guide_forward(pdhgc_guide* g, const __nv_bfloat16* feat, int64_t rows, float
   const long long most = (long long)kTcPerSm * g->max_ctas;
   const long long grid = tiles < most ? tiles : most;
   k_guide_forward_tc<<<(unsigned)grid, kTcRows, sizeof(TcSmem), st>>>(g->wb, g->w, feat, (long long)rows, p, g->err,
-                                                                      g->tc_wait_limit);
+                                                                      g->wait_limit);
 #else
   const long long tiles = (rows + 15) / 16;
   long long grid = (tiles + kGWarps - 1) / kGWarps;
@@ -1173,6 +1174,7 @@ int pdhgc_guide_train(pdhgc_guide* g, const uint16_t* feat, const uint8_t* label
   const int grid = nchunks < g->max_ctas ? nchunks : g->max_ctas;
   const GuideBatch B{reinterpret_cast<const __nv_bfloat16*>(feat), labels, (long long)rows, nullptr, batch,
                      (unsigned long long)seed};
+  const int limit = (int)std::min<long long>(g->wait_limit, kTrainWaitLimit);
   std::vector<float2> c;
   for (int64_t s0 = 0; s0 < steps; s0 += kTrainSteps) {
     const int n = (int)(steps - s0 < kTrainSteps ? steps - s0 : kTrainSteps);
@@ -1195,7 +1197,7 @@ int pdhgc_guide_train(pdhgc_guide* g, const uint16_t* feat, const uint8_t* label
     cfg.attrs = attr;
     cfg.numAttrs = 1;
     GK(cudaLaunchKernelEx(&cfg, k_guide_train, g->wb, g->w, B, (long long)s0, n, g->partials, g->grad, g->m1, g->m2, lr,
-                          (const float2*)coef, hist, bar, g->err));
+                          (const float2*)coef, hist, bar, g->err, limit));
     g->launches++;
     if (losses) GK(cudaMemcpyAsync(losses + s0, hist, sizeof(float) * (size_t)n, cudaMemcpyDeviceToHost, g->stream));
     rc = guide_check_error(g, g->stream);  // also: c and hist are free again
@@ -1208,7 +1210,7 @@ int64_t pdhgc_guide_kernel_launches(const pdhgc_guide* g) { return g ? g->launch
 
 int pdhgc_guide_set_wait_limit(pdhgc_guide* g, int64_t polls) {
   if (!g || polls < 0) return set_error_detail(PDHGC_ERR_INVALID_ARG, "g is NULL or polls < 0");
-  g->tc_wait_limit = polls > 0 ? polls : 0;
+  g->wait_limit = polls > 0 ? polls : 0;
   return PDHGC_OK;
 }
 

@@ -44,7 +44,7 @@ struct pdhgc_guide {
   int32_t* idx = nullptr;     // explicit minibatch indices (gradient check)
   float* train_buf = nullptr;  // of the training kernel, allocated on first use
   int* err = nullptr;         // set by a kernel whose bounded wait ran out (mapped host memory)
-  long long tc_wait_limit = 1ll << 24;  // polls of a tensor-core completion wait before it gives up
+  long long wait_limit = 1ll << 24;  // polls of a kernel's wait before it gives up (pdhgc_guide_set_wait_limit)
   int idx_cap = 0;
   int64_t adam_t = 0;         // Adam steps taken
   int64_t launches = 0;
