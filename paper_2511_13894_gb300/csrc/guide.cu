@@ -543,9 +543,10 @@ __device__ __forceinline__ float load_samples(TrainSmem& s, const GuideBatch& B,
 }
 
 // the CTA's partial gradient (and loss) of one step over its chunks
-// blockIdx.x, blockIdx.x + gridDim.x, ...; the first one's samples are loaded
+// blockIdx.x, blockIdx.x + nparts, ...; the first one's samples are loaded
 __device__ __forceinline__ void grad_cta(TrainSmem& s, const GuideBf16* __restrict__ wb, const float* __restrict__ w,
-                                         const GuideBatch& B, long long step, float lab, float* __restrict__ out) {
+                                         const GuideBatch& B, long long step, float lab, int nparts,
+                                         float* __restrict__ out) {
   const int batch = B.batch;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, g = lane >> 2, t = lane & 3;
   const uint32_t* sx = reinterpret_cast<const uint32_t*>(s.x);
@@ -574,7 +575,7 @@ __device__ __forceinline__ void grad_cta(TrainSmem& s, const GuideBf16* __restri
 #pragma unroll
   for (int nt = 0; nt < 4; ++nt) gW1[nt][0] = gW1[nt][1] = gW1[nt][2] = gW1[nt][3] = 0.0f;
   const int nchunks = (batch + kChunk - 1) / kChunk;
-  for (int c = blockIdx.x; c < nchunks; c += gridDim.x) {
+  for (int c = blockIdx.x; c < nchunks; c += nparts) {
     const int s_base = c * kChunk + warp * 16;
     if (c != (int)blockIdx.x) lab = load_samples(s, B, step, c);
     const float y0 = __shfl_sync(0xffffffffu, lab, g), y1 = __shfl_sync(0xffffffffu, lab, g + 8);
@@ -756,7 +757,7 @@ __global__ void __launch_bounds__(kGThreads) k_guide_grad(const GuideBf16* __res
   extern __shared__ __align__(16) unsigned char smem_raw[];
   TrainSmem& s = *reinterpret_cast<TrainSmem*>(smem_raw);
   const float lab = load_samples(s, B, step, blockIdx.x);
-  grad_cta(s, wb, w, B, step, lab, partials + (size_t)blockIdx.x * kGPartial);
+  grad_cta(s, wb, w, B, step, lab, gridDim.x, partials + (size_t)blockIdx.x * kGPartial);
 }
 
 // BF16 copy of parameter p of the packed vector
@@ -776,6 +777,7 @@ __device__ __forceinline__ void write_bf16(GuideBf16* wb, int p, float v) {
 
 constexpr int kFoldBatch = 32;
 constexpr int kFoldThreads = 64;  // per CTA: the parameters spread over 87 SMs
+constexpr int kTrainFoldCtas = (kGPartial + kGThreads - 1) / kGThreads;  // a thread per parameter
 // parameter p: fold the per-CTA partials in CTA order; lr > 0: one Adam step
 // (Kingma & Ba 2015, beta1 = 0.9, beta2 = 0.999, eps = 1e-8) with the bias
 // corrections c1 = 1 / (1 - beta1^t), c2 = 1 / (1 - beta2^t).  kFoldBatch
@@ -838,28 +840,38 @@ __device__ __forceinline__ void train_barrier(unsigned* bar, unsigned target, in
 }
 
 // `steps` training steps in one cooperative launch: gradient, barrier, fold and
-// Adam (the parameters spread over the CTAs), barrier.  Two launches per step
-// took 22.5 us (80k rows, batches of 4096), most of it latency; here a step
-// takes 11.6: the next step's samples are read while the barrier is waited for.  coef: (c1, c2) of each step; bar: 0 at launch.
+// Adam (the parameters spread over the CTAs), barrier.  The first nparts CTAs
+// take the gradient, the others (none with kAll) only fold: they are a variant
+// of their own since the test for them costs the large batches 1.2 us a step
+// (4096 rows: 10.5 and 11.7).  Two launches per step took 22.5 us (80k rows,
+// batches of 4096), most of it latency; here a step takes 11.6: the next step's
+// samples are read while the barrier is waited for.  coef: (c1, c2) of each
+// step; bar: 0 at launch.
+template <bool kAll>
 __global__ void __launch_bounds__(kGThreads) k_guide_train(GuideBf16* wb, float* w, GuideBatch B, long long step0,
-                                                           int steps, float* partials, float* grad, float* m1,
-                                                           float* m2, float lr, const float2* __restrict__ coef,
-                                                           float* loss_hist, unsigned* bar, int* err, int limit) {
+                                                           int steps, int n_grad, float* partials, float* grad,
+                                                           float* m1, float* m2, float lr,
+                                                           const float2* __restrict__ coef, float* loss_hist,
+                                                           unsigned* bar, int* err, int limit) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   TrainSmem& s = *reinterpret_cast<TrainSmem*>(smem_raw);
   const int per = (kGPartial + gridDim.x - 1) / gridDim.x;
   const int p0 = blockIdx.x * per, p1 = min(p0 + per, kGPartial);
+  const int nparts = kAll ? (int)gridDim.x : n_grad;
+  const bool has_part = kAll || (int)blockIdx.x < nparts;
   bool failed = false;
   unsigned target = 0;
-  float lab = load_samples(s, B, step0, blockIdx.x);
+  float lab = has_part ? load_samples(s, B, step0, blockIdx.x) : 0.0f;
   for (int k = 0; k < steps; ++k) {
-    grad_cta(s, wb, w, B, step0 + k, lab, partials + (size_t)blockIdx.x * kGPartial);
-    __syncthreads();  // the staged samples are used up
-    if (k + 1 < steps) lab = load_samples(s, B, step0 + k + 1, blockIdx.x);
+    if (has_part) {
+      grad_cta(s, wb, w, B, step0 + k, lab, nparts, partials + (size_t)blockIdx.x * kGPartial);
+      __syncthreads();  // the staged samples are used up
+      if (k + 1 < steps) lab = load_samples(s, B, step0 + k + 1, blockIdx.x);
+    }
     train_barrier(bar, target += gridDim.x, err, limit, failed);
     const float2 c = coef[k];
     for (int p = p0 + (int)threadIdx.x; p < p1; p += kGThreads)
-      fold_param(partials, gridDim.x, p, grad, w, m1, m2, wb, lr, c.x, c.y, loss_hist + k);
+      fold_param(partials, nparts, p, grad, w, m1, m2, wb, lr, c.x, c.y, loss_hist + k);
     if (k + 1 < steps) train_barrier(bar, target += gridDim.x, err, limit, failed);
   }
 }
@@ -1165,13 +1177,19 @@ int pdhgc_guide_train(pdhgc_guide* g, const uint16_t* feat, const uint8_t* label
   if (rc != PDHGC_OK) return rc;
   if (!g->train_buf) {  // kept by the handle: (c1, c2) and the loss of each step of a launch, the barrier counter
     GK(cudaMalloc(&g->train_buf, sizeof(float) * 3 * kTrainSteps + sizeof(unsigned)));
-    GK(cudaFuncSetAttribute(k_guide_train, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)train_smem()));
+    GK(cudaFuncSetAttribute(k_guide_train<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)train_smem()));
+    GK(cudaFuncSetAttribute(k_guide_train<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)train_smem()));
   }
   float2* const coef = reinterpret_cast<float2*>(g->train_buf);
   float* const hist = g->train_buf + 2 * kTrainSteps;
   unsigned* const bar = reinterpret_cast<unsigned*>(g->train_buf + 3 * kTrainSteps);
   const int nchunks = (batch + kChunk - 1) / kChunk;
-  const int grid = nchunks < g->max_ctas ? nchunks : g->max_ctas;
+  const int nparts = std::min(nchunks, g->max_ctas);
+  // the fold takes a thread per parameter where the gradient has fewer CTAs; on
+  // the gradient's CTAs alone (one for up to 64 rows) a step took 45 us at 64
+  // rows (now 10.2; two launches 15), 32 at 128 (10.7), 16 at 512 (10.9) and
+  // 11.1 at 2048 (11.0)
+  const int grid = std::min(std::max(nparts, kTrainFoldCtas), g->max_ctas);
   const GuideBatch B{reinterpret_cast<const __nv_bfloat16*>(feat), labels, (long long)rows, nullptr, batch,
                      (unsigned long long)seed};
   const int limit = (int)std::min<long long>(g->wait_limit, kTrainWaitLimit);
@@ -1196,8 +1214,9 @@ int pdhgc_guide_train(pdhgc_guide* g, const uint16_t* feat, const uint8_t* label
     cfg.stream = g->stream;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
-    GK(cudaLaunchKernelEx(&cfg, k_guide_train, g->wb, g->w, B, (long long)s0, n, g->partials, g->grad, g->m1, g->m2, lr,
-                          (const float2*)coef, hist, bar, g->err, limit));
+    GK(cudaLaunchKernelEx(&cfg, nparts == grid ? k_guide_train<true> : k_guide_train<false>, g->wb, g->w, B,
+                          (long long)s0, n, nparts, g->partials, g->grad, g->m1, g->m2, lr, (const float2*)coef, hist, bar,
+                          g->err, limit));
     g->launches++;
     if (losses) GK(cudaMemcpyAsync(losses + s0, hist, sizeof(float) * (size_t)n, cudaMemcpyDeviceToHost, g->stream));
     rc = guide_check_error(g, g->stream);  // also: c and hist are free again
