@@ -87,11 +87,23 @@ __device__ __forceinline__ unsigned long long mix64(unsigned long long seed, uns
   return z ^ (z >> 31);
 }
 
+// Loads from L2 of what other CTAs of the training kernel write between its
+// barriers: volatile, so that none is kept from one step for the next
+__device__ __forceinline__ float ld_l2(const float* p) {
+  float v;
+  asm volatile("ld.global.cg.f32 %0, [%1];" : "=f"(v) : "l"(p));
+  return v;
+}
+__device__ __forceinline__ uint4 ld_l2(const uint4* p) {
+  uint4 v;
+  asm volatile("ld.global.cg.v4.u32 {%0, %1, %2, %3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "l"(p));
+  return v;
+}
+
 // stage W1 (padded, stride 40) and W2 (stride 72) and optionally W2' in shared
 // memory, 16 bytes a load: all of a thread's loads are in flight together (10
 // in the training kernel; one word each, 40 in batches, took several times
-// the latency of L2).  From L2: a training kernel may start before the update
-// of the weights it reads has ended, beside CTAs that hold the old ones in L1
+// the latency of L2)
 __device__ void stage_weights(const GuideBf16* __restrict__ wb, __nv_bfloat16* sW1, __nv_bfloat16* sW2,
                               __nv_bfloat16* sW2T) {
   static_assert(kGFeat == 32 && kGHid == 64 && kS40 % 8 == 0 && kS72 % 8 == 0, "16-byte pieces of rows");
@@ -106,12 +118,12 @@ __device__ void stage_weights(const GuideBf16* __restrict__ wb, __nv_bfloat16* s
   const int tid = threadIdx.x;
   uint4 v1[N1], v2[N2], v3[N2];
 #pragma unroll
-  for (int i = 0; i < N1; ++i) v1[i] = __ldcg(w1 + tid + i * kGThreads);
+  for (int i = 0; i < N1; ++i) v1[i] = ld_l2(w1 + tid + i * kGThreads);
 #pragma unroll
-  for (int i = 0; i < N2; ++i) v2[i] = __ldcg(w2 + tid + i * kGThreads);
+  for (int i = 0; i < N2; ++i) v2[i] = ld_l2(w2 + tid + i * kGThreads);
   if (sW2T)
 #pragma unroll
-    for (int i = 0; i < N2; ++i) v3[i] = __ldcg(w2t + tid + i * kGThreads);
+    for (int i = 0; i < N2; ++i) v3[i] = ld_l2(w2t + tid + i * kGThreads);
 #pragma unroll
   for (int i = 0; i < N1; ++i) {
     const int e = tid + i * kGThreads;
@@ -551,21 +563,37 @@ __device__ __forceinline__ void grad_cta(TrainSmem& s, const GuideBf16* __restri
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, g = lane >> 2, t = lane & 3;
   const uint32_t* sx = reinterpret_cast<const uint32_t*>(s.x);
   stage_weights(wb, s.w1, s.w2, s.w2t);
-  for (int j = threadIdx.x; j < kGHid; j += blockDim.x) {
-    s.b1[j] = __ldcg(w + kOffB1 + j);
-    s.b2[j] = __ldcg(w + kOffB2 + j);
-    s.w3[j] = __bfloat162float(__ldcg(wb->w3 + j));
+  // issued together: one latency of L2
+  const int tid = threadIdx.x;
+  float b1 = 0.0f, b2 = 0.0f;
+  uint4 w3 = make_uint4(0u, 0u, 0u, 0u);
+  if (tid < kGHid) {
+    b1 = ld_l2(w + kOffB1 + tid);
+    b2 = ld_l2(w + kOffB2 + tid);
+  }
+  if (tid < kGHid / 8) w3 = ld_l2(reinterpret_cast<const uint4*>(wb->w3) + tid);
+  const float b3 = ld_l2(w + kOffB3);
+  if (tid < kGHid) {
+    s.b1[tid] = b1;
+    s.b2[tid] = b2;
     for (int q = 0; q < kGWarps; ++q) {
-      s.gb1[q][j] = 0.0f;
-      s.gb2[q][j] = 0.0f;
-      s.gw3[q][j] = 0.0f;
+      s.gb1[q][tid] = 0.0f;
+      s.gb2[q][tid] = 0.0f;
+      s.gw3[q][tid] = 0.0f;
+    }
+  }
+  if (tid < kGHid / 8) {
+    const uint32_t pair[4] = {w3.x, w3.y, w3.z, w3.w};
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {  // a BF16 value is the upper half of its FP32 bits
+      s.w3[8 * tid + 2 * u] = __uint_as_float(pair[u] << 16);
+      s.w3[8 * tid + 2 * u + 1] = __uint_as_float(pair[u] & 0xffff0000u);
     }
   }
   if (threadIdx.x < kGWarps) {
     s.gb3[threadIdx.x] = 0.0f;
     s.loss[threadIdx.x] = 0.0f;
   }
-  const float b3 = __ldcg(w + kOffB3);
   const float inv_b = 1.0f / (float)batch;
   __syncthreads();
   const uint32_t* sw2t = reinterpret_cast<const uint32_t*>(s.w2t);
@@ -791,7 +819,7 @@ __device__ __forceinline__ void fold_param(const float* __restrict__ partials, i
   for (int b0 = 0; b0 < nparts; b0 += kFoldBatch) {
     float v[kFoldBatch];
 #pragma unroll
-    for (int u = 0; u < kFoldBatch; ++u) v[u] = __ldcg(partials + (size_t)min(b0 + u, nparts - 1) * kGPartial + p);
+    for (int u = 0; u < kFoldBatch; ++u) v[u] = ld_l2(partials + (size_t)min(b0 + u, nparts - 1) * kGPartial + p);
 #pragma unroll
     for (int u = 0; u < kFoldBatch; ++u)
       if (b0 + u < nparts) gsum += v[u];
@@ -802,11 +830,11 @@ __device__ __forceinline__ void fold_param(const float* __restrict__ partials, i
     return;
   }
   if (lr > 0.0f) {
-    const float a = 0.9f * __ldcg(m1 + p) + 0.1f * gsum;
-    const float v = 0.999f * __ldcg(m2 + p) + 0.001f * gsum * gsum;
+    const float a = 0.9f * ld_l2(m1 + p) + 0.1f * gsum;
+    const float v = 0.999f * ld_l2(m2 + p) + 0.001f * gsum * gsum;
     m1[p] = a;
     m2[p] = v;
-    const float wn = __ldcg(w + p) - lr * (a * c1) / (sqrtf(v * c2) + 1e-8f);
+    const float wn = ld_l2(w + p) - lr * (a * c1) / (sqrtf(v * c2) + 1e-8f);
     w[p] = wn;
     write_bf16(wb, p, wn);
   }
