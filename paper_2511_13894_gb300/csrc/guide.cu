@@ -780,12 +780,12 @@ __device__ __forceinline__ void grad_cta(TrainSmem& s, const GuideBf16* __restri
 }
 
 __global__ void __launch_bounds__(kGThreads) k_guide_grad(const GuideBf16* __restrict__ wb,
-                                                           const float* __restrict__ w, GuideBatch B, long long step,
+                                                           const float* __restrict__ w, GuideBatch B,
                                                            float* __restrict__ partials) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   TrainSmem& s = *reinterpret_cast<TrainSmem*>(smem_raw);
-  const float lab = load_samples(s, B, step, blockIdx.x);
-  grad_cta(s, wb, w, B, step, lab, gridDim.x, partials + (size_t)blockIdx.x * kGPartial);
+  const float lab = load_samples(s, B, 0, blockIdx.x);
+  grad_cta(s, wb, w, B, 0, lab, gridDim.x, partials + (size_t)blockIdx.x * kGPartial);
 }
 
 // BF16 copy of parameter p of the packed vector
@@ -806,15 +806,10 @@ __device__ __forceinline__ void write_bf16(GuideBf16* wb, int p, float v) {
 constexpr int kFoldBatch = 32;
 constexpr int kFoldThreads = 64;  // per CTA: the parameters spread over 87 SMs
 constexpr int kTrainFoldCtas = (kGPartial + kGThreads - 1) / kGThreads;  // a thread per parameter
-// parameter p: fold the per-CTA partials in CTA order; lr > 0: one Adam step
-// (Kingma & Ba 2015, beta1 = 0.9, beta2 = 0.999, eps = 1e-8) with the bias
-// corrections c1 = 1 / (1 - beta1^t), c2 = 1 / (1 - beta2^t).  kFoldBatch
-// partials are in flight (one after another in fours, 64 cost 16 latencies of
-// L2); all reads from L2: in the training kernel other CTAs wrote them
-__device__ __forceinline__ void fold_param(const float* __restrict__ partials, int nparts, int p,
-                                           float* __restrict__ grad, float* __restrict__ w, float* __restrict__ m1,
-                                           float* __restrict__ m2, GuideBf16* __restrict__ wb, float lr, float c1,
-                                           float c2, float* __restrict__ loss_hist) {
+// gradient p (kGParams: the loss): the per-CTA partials in CTA order.
+// kFoldBatch of them are in flight (one after another in fours, 64 cost 16
+// latencies of L2)
+__device__ __forceinline__ float fold_param(const float* __restrict__ partials, int nparts, int p) {
   float gsum = 0.0f;
   for (int b0 = 0; b0 < nparts; b0 += kFoldBatch) {
     float v[kFoldBatch];
@@ -824,27 +819,27 @@ __device__ __forceinline__ void fold_param(const float* __restrict__ partials, i
     for (int u = 0; u < kFoldBatch; ++u)
       if (b0 + u < nparts) gsum += v[u];
   }
-  grad[p] = gsum;
-  if (p == kGParams) {
-    if (loss_hist) *loss_hist = gsum;
-    return;
-  }
-  if (lr > 0.0f) {
-    const float a = 0.9f * ld_l2(m1 + p) + 0.1f * gsum;
-    const float v = 0.999f * ld_l2(m2 + p) + 0.001f * gsum * gsum;
-    m1[p] = a;
-    m2[p] = v;
-    const float wn = ld_l2(w + p) - lr * (a * c1) / (sqrtf(v * c2) + 1e-8f);
-    w[p] = wn;
-    write_bf16(wb, p, wn);
-  }
+  return gsum;
 }
 
-__global__ void k_guide_fold(const float* __restrict__ partials, int nparts, float* __restrict__ grad,
-                             float* __restrict__ w, float* __restrict__ m1, float* __restrict__ m2,
-                             GuideBf16* __restrict__ wb, float lr, float c1, float c2) {
+__global__ void k_guide_fold(const float* __restrict__ partials, int nparts, float* __restrict__ grad) {
   const int p = blockIdx.x * blockDim.x + threadIdx.x;
-  if (p < kGPartial) fold_param(partials, nparts, p, grad, w, m1, m2, wb, lr, c1, c2, nullptr);
+  if (p < kGPartial) grad[p] = fold_param(partials, nparts, p);
+}
+
+// one Adam step of parameter p (Kingma & Ba 2015, beta1 = 0.9, beta2 = 0.999,
+// eps = 1e-8) with the bias corrections c1 = 1 / (1 - beta1^t), c2 = 1 / (1 -
+// beta2^t), and its BF16 copy
+__device__ __forceinline__ void adam_param(int p, float gsum, float* __restrict__ w, float* __restrict__ m1,
+                                           float* __restrict__ m2, GuideBf16* __restrict__ wb, float lr, float c1,
+                                           float c2) {
+  const float a = 0.9f * ld_l2(m1 + p) + 0.1f * gsum;
+  const float v = 0.999f * ld_l2(m2 + p) + 0.001f * gsum * gsum;
+  m1[p] = a;
+  m2[p] = v;
+  const float wn = ld_l2(w + p) - lr * (a * c1) / (sqrtf(v * c2) + 1e-8f);
+  w[p] = wn;
+  write_bf16(wb, p, wn);
 }
 
 // all CTAs of a cooperative grid meet; a wait that runs out sets the error
@@ -877,10 +872,9 @@ __device__ __forceinline__ void train_barrier(unsigned* bar, unsigned target, in
 // step; bar: 0 at launch.
 template <bool kAll>
 __global__ void __launch_bounds__(kGThreads) k_guide_train(GuideBf16* wb, float* w, GuideBatch B, long long step0,
-                                                           int steps, int n_grad, float* partials, float* grad,
-                                                           float* m1, float* m2, float lr,
-                                                           const float2* __restrict__ coef, float* loss_hist,
-                                                           unsigned* bar, int* err, int limit) {
+                                                           int steps, int n_grad, float* partials, float* m1,
+                                                           float* m2, float lr, const float2* __restrict__ coef,
+                                                           float* loss_hist, unsigned* bar, int* err, int limit) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   TrainSmem& s = *reinterpret_cast<TrainSmem*>(smem_raw);
   const int per = (kGPartial + gridDim.x - 1) / gridDim.x;
@@ -898,8 +892,13 @@ __global__ void __launch_bounds__(kGThreads) k_guide_train(GuideBf16* wb, float*
     }
     train_barrier(bar, target += gridDim.x, err, limit, failed);
     const float2 c = coef[k];
-    for (int p = p0 + (int)threadIdx.x; p < p1; p += kGThreads)
-      fold_param(partials, nparts, p, grad, w, m1, m2, wb, lr, c.x, c.y, loss_hist + k);
+    for (int p = p0 + (int)threadIdx.x; p < p1; p += kGThreads) {
+      const float gsum = fold_param(partials, nparts, p);
+      if (p == kGParams)
+        loss_hist[k] = gsum;
+      else
+        adam_param(p, gsum, w, m1, m2, wb, lr, c.x, c.y);
+    }
     if (k + 1 < steps) train_barrier(bar, target += gridDim.x, err, limit, failed);
   }
 }
@@ -959,23 +958,15 @@ int guide_check_error(pdhgc_guide* g, cudaStream_t st) {
   return PDHGC_OK;
 }
 
-int guide_step(pdhgc_guide* g, const __nv_bfloat16* feat, const uint8_t* labels, int64_t rows, const int32_t* idx,
-               int batch, uint64_t seed, int64_t step, float adam_lr, cudaStream_t st) {
+int guide_gradient(pdhgc_guide* g, const __nv_bfloat16* feat, const uint8_t* labels, int64_t rows, const int32_t* idx,
+                   int batch, cudaStream_t st) {
   const int nchunks = (batch + kChunk - 1) / kChunk;
-  const int grid = nchunks < g->max_ctas ? nchunks : g->max_ctas;
+  const int grid = std::min(nchunks, g->max_ctas);
   k_guide_grad<<<grid, kGThreads, train_smem(), st>>>(
-      g->wb, g->w, GuideBatch{feat, labels, (long long)rows, idx, batch, (unsigned long long)seed}, (long long)step,
-      g->partials);
+      g->wb, g->w, GuideBatch{feat, labels, (long long)rows, idx, batch, 0}, g->partials);
   g->launches++;
   GKL();
-  float c1 = 0.0f, c2 = 0.0f;
-  if (adam_lr > 0.0f) {
-    g->adam_t++;
-    c1 = (float)(1.0 / (1.0 - std::pow(0.9, (double)g->adam_t)));
-    c2 = (float)(1.0 / (1.0 - std::pow(0.999, (double)g->adam_t)));
-  }
-  k_guide_fold<<<(kGPartial + kFoldThreads - 1) / kFoldThreads, kFoldThreads, 0, st>>>(g->partials, grid, g->grad, g->w, g->m1, g->m2, g->wb,
-                                                        adam_lr, c1, c2);
+  k_guide_fold<<<(kGPartial + kFoldThreads - 1) / kFoldThreads, kFoldThreads, 0, st>>>(g->partials, grid, g->grad);
   g->launches++;
   GKL();
   return PDHGC_OK;
@@ -1186,8 +1177,7 @@ int pdhgc_guide_grad(pdhgc_guide* g, const uint16_t* feat, const uint8_t* labels
     g->idx_cap = batch;
   }
   GK(cudaMemcpyAsync(g->idx, idx, sizeof(int32_t) * (size_t)batch, cudaMemcpyHostToDevice, g->stream));
-  rc = guide_step(g, reinterpret_cast<const __nv_bfloat16*>(feat), labels, rows, g->idx, batch, 0, 0, 0.0f,
-                  g->stream);
+  rc = guide_gradient(g, reinterpret_cast<const __nv_bfloat16*>(feat), labels, rows, g->idx, batch, g->stream);
   if (rc != PDHGC_OK) return rc;
   std::vector<float> h(kGPartial);
   GK(cudaMemcpyAsync(h.data(), g->grad, sizeof(float) * kGPartial, cudaMemcpyDeviceToHost, g->stream));
@@ -1243,7 +1233,7 @@ int pdhgc_guide_train(pdhgc_guide* g, const uint16_t* feat, const uint8_t* label
     cfg.attrs = attr;
     cfg.numAttrs = 1;
     GK(cudaLaunchKernelEx(&cfg, nparts == grid ? k_guide_train<true> : k_guide_train<false>, g->wb, g->w, B,
-                          (long long)s0, n, nparts, g->partials, g->grad, g->m1, g->m2, lr, (const float2*)coef, hist, bar,
+                          (long long)s0, n, nparts, g->partials, g->m1, g->m2, lr, (const float2*)coef, hist, bar,
                           g->err, limit));
     g->launches++;
     if (losses) GK(cudaMemcpyAsync(losses + s0, hist, sizeof(float) * (size_t)n, cudaMemcpyDeviceToHost, g->stream));

@@ -59,11 +59,9 @@ int guide_forward(pdhgc_guide* g, const __nv_bfloat16* feat, int64_t rows, float
 // the error word of the network's kernels (synchronises st); DEVICE when set
 int guide_check_error(pdhgc_guide* g, cudaStream_t st);
 
-// one minibatch gradient (idx != nullptr: explicit device indices; else drawn
-// from SplitMix64(seed, step * batch + s) mod rows) folded into g->grad;
-// adam_lr > 0 also applies one Adam step
-int guide_step(pdhgc_guide* g, const __nv_bfloat16* feat, const uint8_t* labels, int64_t rows,
-               const int32_t* idx, int batch, uint64_t seed, int64_t step, float adam_lr, cudaStream_t st);
+// the gradient of one minibatch (idx: device indices of its rows) folded into g->grad
+int guide_gradient(pdhgc_guide* g, const __nv_bfloat16* feat, const uint8_t* labels, int64_t rows,
+                   const int32_t* idx, int batch, cudaStream_t st);
 
 // refresh the BF16 copies from the FP32 master parameters
 int guide_sync_bf16(pdhgc_guide* g, cudaStream_t st);
