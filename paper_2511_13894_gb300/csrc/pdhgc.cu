@@ -258,7 +258,7 @@ struct PhaseInit {
 __global__ void k_init_scalars(Scalars* S, PhaseInit pi, const double* cc2, unsigned* seq) {
   if (threadIdx.x != 0) return;
   seq[kStepBar] = 0u;
-  seq[0] += 1u;  // no step has number 0
+  seq[0] = 1u;  // the entries of the step kernel are cleared to 0
   S->eps_rel = pi.eps_rel;
   S->beta_suff = pi.beta_suff;
   S->beta_nec = pi.beta_nec;
@@ -749,6 +749,7 @@ struct pdhgc_lp {
     size_t smem = 0;
     // (value, step) entries of x_bar and y; of this precision only: bits of the other's values would be read as steps
     void *fx = nullptr, *fy = nullptr;
+    size_t entry_bytes = 0;  // of both, fx first
   } steps64, steps32;
   bool step_flow = false;
   int step_ctas = 0;
@@ -1071,10 +1072,10 @@ int setup_steps_one(pdhgc_lp* lp, pdhgc_lp::Steps& sp, const Csr& A, const Csr& 
     q.col = reinterpret_cast<int*>(d_room + off[t].col);
     q.val = d_room + off[t].val;
   }
-  if (lp->step_flow) {  // no entry is of a step yet
-    CK(cudaMemsetAsync(d_room + fx, 0, room - fx, st));
+  if (lp->step_flow) {
     sp.fx = d_room + fx;
     sp.fy = d_room + fy;
+    sp.entry_bytes = room - fx;
   }
   RET(fill_steps<VT>(lp, sp, true, st));
   CK(cudaStreamSynchronize(st));  // the plans go out of scope
@@ -1466,6 +1467,10 @@ int run_phase(pdhgc_lp* lp, const DevModel& md, const DevModel32& md32, const Ph
                        lp->it32.xlo, lp->it32.ylo, lp->it32.xa,   lp->it32.ya};
   k_init_iterates<<<gnm, 256, 0, st>>>(n, m, md, lp->it, x_start, w32, y_start);
   k_init_scalars<<<1, 32, 0, st>>>(lp->S, pi, cc2, lp->step_seq);
+  // steps are numbered from the phase's start, and every step writes every
+  // entry: no entry is ever more than a chunk of steps behind
+  const pdhgc_lp::Steps& sp = fp32 ? lp->steps32 : lp->steps64;
+  if (sp.entry_bytes > 0) CK(cudaMemsetAsync(sp.fx, 0, sp.entry_bytes, st));
   lp->launches += 2;
   CKL();
   // phase 1 records its restart history (start point and restart points)

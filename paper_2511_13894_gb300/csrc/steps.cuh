@@ -59,7 +59,7 @@ struct StepEntry<float> {
 struct StepFlow {
   void* fy;             // m entries: y, gathered by the pass over A'
   void* fx;             // n entries: x_bar, gathered by the pass over A
-  const unsigned* seq;  // number of this launch's first step; grows from launch to launch
+  const unsigned* seq;  // number of this launch's first step; 1 at a phase's start, where all entries are 0
   unsigned* bar;        // barrier mode: arrivals, 0 at launch
   int* err;             // set when a bounded wait ran out
   int limit;            // polls of one wait before that
