@@ -23,9 +23,8 @@
 //     are copied to shared memory once per CTA and pass.
 // Loop time per iteration, before (two launches) and now, us (GB300, Halpern):
 //   FP64  200 x 500 random face 7.9 -> 3.4 (flow), 5000 x 17500 with bounds
-//         (averaged) 10.3 -> 5.1 (flow), 2000 x 8000 power law 13.8 -> 6.8 to 8.9
-//         (flow; it depends on where the entries lie in L2), 20k x 80k power law
-//         18.7 -> 12.7 (barrier)
+//         (averaged) 10.3 -> 5.1 (flow), 2000 x 8000 power law 13.8 -> 7.9
+//         (barrier), 20k x 80k power law 18.7 -> 12.7 (barrier)
 //   FP32  20k x 80k power law (averaged) 17.7 -> 12.4 (barrier)
 #pragma once
 #include "kernels.cuh"
@@ -108,7 +107,7 @@ __device__ __forceinline__ float ld_iter(const float* p) {
 }
 
 // Pairs of steps whose gathers a lane keeps in flight.  FP64 tasks are short (4
-// to 8 steps): 4 pairs instead of 2 measured 14.1 against 12.8 us per iteration
+// to 8 steps on the LPs measured, kStepMaxCols at most): 4 pairs instead of 2 measured 14.1 against 12.8 us per iteration
 // on the 20k x 80k power law.  FP32 tasks have up to 32 steps in SELL rows and
 // 128 in long ones: 8 pairs (4 in flow order, whose entries take twice the
 // registers) are what 128 registers hold without spilling.
