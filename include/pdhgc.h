@@ -16,7 +16,8 @@
  *  - All device work is enqueued on the CUDA stream given to
  *    pdhgc_lp_create (NULL = the legacy default stream).  Calls that return
  *    host results synchronise that stream before returning.
- *  - A handle is not thread-safe; different handles are independent.
+ *  - A handle is not thread-safe; different handles are independent (several
+ *    at work on one GPU at a time: pdhgc_set_gpu_sharing).
  *  - Vectors are dense, in the user's row / column order, FP64.  A pointer
  *    argument documented "host or device" is a device pointer when the
  *    call's `on_device` flag is 1 and a host pointer when it is 0.
@@ -308,6 +309,38 @@ int pdhgc_set_primal_layout(pdhgc_lp* lp, int32_t chunked);
 #define PDHGC_LAUNCH_GRAPH  0
 #define PDHGC_LAUNCH_STREAM 1
 int pdhgc_set_launch_mode(pdhgc_lp* lp, int32_t mode);
+
+/*
+ * pdhgc_set_gpu_sharing — whether other handles are at work on the GPU at the
+ * same time.  0 (the default): an LP whose matrix entries fit in the SMs'
+ * shared memory runs its loop and power iteration as one kernel per check
+ * period, a cooperative grid of up to a CTA on every SM, which starts only when
+ * all of its CTAs fit: handles at work in several threads take turns.  1: the
+ * handle uses the kernels of larger LPs (a launch per matrix pass), which run
+ * side by side.  One handle alone is 1.7 to 2.4 times slower with them, two
+ * together about as fast, four of a 2000 x 8000 LP in four threads 1.8 times
+ * faster (4096 iterations each: 128 -> 71 ms) and four of a 5000 x 17500 LP 1.5
+ * times (77 -> 52 ms); four LPs that leave SMs free (200 x 500) 2.3 times slower
+ * (16 -> 37 ms).  The FP64 row sums have another order, so results differ in
+ * rounding.  Takes effect at the next phase.  A choice of schedule (the paper
+ * has no counterpart).  Errors: INVALID_ARG.
+ */
+int pdhgc_set_gpu_sharing(pdhgc_lp* lp, int32_t shared);
+
+/*
+ * pdhgc_get_loop_kernel — what the handle's next phase in `precision` runs
+ * its loop on, with the inner loop of the last pdhgc_solve:
+ *   PDHGC_LOOP_PASSES  (0): a launch per matrix pass;
+ *   PDHGC_LOOP_BARRIER (1): a launch per check period, a grid barrier after
+ *     each pass;
+ *   PDHGC_LOOP_FLOW    (2): the same without barriers, each gather waiting for
+ *     the values it reads.
+ * A query for measurement and tests.  Errors: INVALID_ARG.
+ */
+#define PDHGC_LOOP_PASSES  0
+#define PDHGC_LOOP_BARRIER 1
+#define PDHGC_LOOP_FLOW    2
+int pdhgc_get_loop_kernel(const pdhgc_lp* lp, int32_t precision, int32_t* kernel);
 
 /*
  * pdhgc_set_wait_limit — polls each wait of a kernel whose CTAs wait for each

@@ -752,6 +752,7 @@ struct pdhgc_lp {
     size_t entry_bytes = 0;  // of both, fx first
   } steps64, steps32;
   bool step_flow = false;
+  bool shared_gpu = false;  // pdhgc_set_gpu_sharing: the per-pass kernels, whatever the plans
   int step_ctas = 0;
   size_t step_smem_max = 0;
   unsigned* step_seq = nullptr;  // [0] step number of the next launch, [kStepBar] barrier arrivals
@@ -976,7 +977,7 @@ int launch_steps(pdhgc_lp* lp, const OpT& opT, const OpA& opA, int period, int w
 
 // the loop of this precision and algorithm runs on the step kernel
 bool use_steps(const pdhgc_lp* lp, bool fp32, bool halpern) {
-  return (fp32 ? lp->steps32.on : lp->steps64.on) && !(halpern && lp->chunked_primal);
+  return (fp32 ? lp->steps32.on : lp->steps64.on) && !lp->shared_gpu && !(halpern && lp->chunked_primal);
 }
 
 // the indices (once) or the values of a step layout, from the scaled CSR
@@ -1221,7 +1222,7 @@ int setup_scaling(pdhgc_lp* lp, const pdhgc_params& p) {
   CK(cudaMemsetAsync(&lp->S->pi_zero, 0, sizeof(int), st));
   k_fill<<<grid_for(n), 256, 0, st>>>(lp->pi_v, n, 1.0 / std::sqrt((double)n));
   lp->launches++;
-  if (lp->steps64.on) {
+  if (lp->steps64.on && !lp->shared_gpu) {
     const pdhgc_lp::Steps& sp = lp->steps64;
     double* const part = lp->step_part + lp->step_ctas;
     CK(cudaMemsetAsync(lp->step_seq + kStepBar, 0, sizeof(unsigned), st));
@@ -2873,6 +2874,20 @@ int pdhgc_set_launch_mode(pdhgc_lp* lp, int32_t mode) {
   if (!lp || (mode != PDHGC_LAUNCH_GRAPH && mode != PDHGC_LAUNCH_STREAM))
     return set_err(PDHGC_ERR_INVALID_ARG, "mode must be PDHGC_LAUNCH_GRAPH or PDHGC_LAUNCH_STREAM");
   lp->launch_mode = mode;
+  return PDHGC_OK;
+}
+
+int pdhgc_set_gpu_sharing(pdhgc_lp* lp, int32_t shared) {
+  if (!lp || (shared != 0 && shared != 1)) return set_err(PDHGC_ERR_INVALID_ARG, "shared must be 0 or 1");
+  lp->shared_gpu = shared != 0;
+  return PDHGC_OK;
+}
+
+int pdhgc_get_loop_kernel(const pdhgc_lp* lp, int32_t precision, int32_t* kernel) {
+  if (!lp || !kernel || (precision != PDHGC_FP64 && precision != PDHGC_FP32_BULK))
+    return set_err(PDHGC_ERR_INVALID_ARG, "bad argument");
+  const bool steps = use_steps(lp, precision == PDHGC_FP32_BULK, lp->params.algorithm == PDHGC_ALG_HALPERN);
+  *kernel = !steps ? PDHGC_LOOP_PASSES : lp->step_flow ? PDHGC_LOOP_FLOW : PDHGC_LOOP_BARRIER;
   return PDHGC_OK;
 }
 

@@ -38,6 +38,7 @@ FP64, FP32_BULK = 0, 1
 PHASE1, CORNER, DUAL_CORNER = 0, 1, 2
 AVERAGED, HALPERN = 0, 1  # pdhgc_params.algorithm (PDHGC_ALG_*)
 LAUNCH_GRAPH, LAUNCH_STREAM = 0, 1  # pdhgc_set_launch_mode
+LOOP_PASSES, LOOP_BARRIER, LOOP_FLOW = 0, 1, 2  # pdhgc_get_loop_kernel
 
 
 class PdhgcError(RuntimeError):
@@ -112,6 +113,8 @@ _sig = {
     "pdhgc_get_layout": (C.c_int, [_vp, _vp]),
     "pdhgc_set_primal_layout": (C.c_int, [_vp, C.c_int32]),
     "pdhgc_set_launch_mode": (C.c_int, [_vp, C.c_int32]),
+    "pdhgc_set_gpu_sharing": (C.c_int, [_vp, C.c_int32]),
+    "pdhgc_get_loop_kernel": (C.c_int, [_vp, C.c_int32, _vp]),
     "pdhgc_set_wait_limit": (C.c_int, [_vp, C.c_int64]),
     "pdhgc_uniform": (C.c_int, [C.c_uint64, C.c_int64, C.c_double, _vp, _vp]),
     "pdhgc_kkt_eval": (C.c_int, [C.c_int32, C.c_int32, C.c_int64, _vp, _vp, _vp, _vp, _vp, _vp, _vp, _vp, _vp,
@@ -288,6 +291,16 @@ class LP:
         """pdhgc_set_launch_mode: LAUNCH_GRAPH (default, one conditional graph
         per phase) or LAUNCH_STREAM (plain launches, one body at a time)."""
         _check(lib.pdhgc_set_launch_mode(self._h, int(mode)), "pdhgc_set_launch_mode")
+
+    def set_gpu_sharing(self, shared: bool):
+        """pdhgc_set_gpu_sharing: True when other work runs on the GPU beside this handle's."""
+        _check(lib.pdhgc_set_gpu_sharing(self._h, int(bool(shared))), "pdhgc_set_gpu_sharing")
+
+    def get_loop_kernel(self, precision: int = FP64) -> int:
+        """pdhgc_get_loop_kernel: LOOP_PASSES, LOOP_BARRIER or LOOP_FLOW."""
+        out = C.c_int32(0)
+        _check(lib.pdhgc_get_loop_kernel(self._h, int(precision), C.byref(out)), "pdhgc_get_loop_kernel")
+        return int(out.value)
 
     def set_wait_limit(self, polls: int):
         """pdhgc_set_wait_limit (failure-path tests)."""

@@ -1,4 +1,5 @@
-"""The persistent step kernel outside a plain solve: replayed passes, waits that run out (needs a GB300)."""
+"""The persistent step kernel outside a plain solve: replayed passes, waits that run out, and the per-pass kernels in
+its place (needs a GB300)."""
 import numpy as np
 import pytest
 
@@ -105,4 +106,38 @@ def test_a_wait_that_runs_out_is_reported_by_its_own_call(name, precision):
     g.corner_phase(**ckw)
     for a, b in zip(_results(g), want):
         assert np.array_equal(a, b)
+    g.close()
+
+
+LOOP = {"hot_lengths": P.LOOP_FLOW, "barrier_order": P.LOOP_BARRIER}  # the others: flow
+
+
+@pytest.mark.parametrize("algorithm", ["halpern", "averaged"])
+@pytest.mark.parametrize("name", list(CASES))
+def test_step_kernel_equals_the_per_pass_kernels(name, algorithm):
+    """The same phase (a corner phase: 192 iterations, three checks) on a handle that shares the GPU: in FP32 bulk the
+    step kernel sums every row in the per-pass kernels' order, so all bits are equal; in FP64 the iterates agree to
+    the parity tests' 1e-10."""
+    g = P.lp_from_dict(CASES[name]())
+    for precision in (P.FP64, P.FP32_BULK):
+        g.solve(max_iters=70, eps_rel=-1.0, precision=precision,
+                algorithm=P.HALPERN if algorithm == "halpern" else P.AVERAGED)
+        out = []
+        for shared in (False, True):
+            g.set_gpu_sharing(shared)
+            assert g.get_loop_kernel(precision) == (P.LOOP_PASSES if shared else LOOP.get(name, P.LOOP_FLOW))
+            before = g.kernel_launches()
+            rep = g.corner_phase(obj_seed=3, eps_rel=1e30, min_iters=192)
+            launches = g.kernel_launches() - before
+            it = g.get_iterates()
+            out.append((rep["iters"], rep["restarts"], launches, [it[k] for k in ("x", "y", "x_avg", "y_avg")]))
+        g.set_gpu_sharing(False)
+        (k0, r0, l0, v0), (k1, r1, l1, v1) = out
+        assert k0 == k1 == 192 and r0 == r1
+        assert l1 - l0 == 192 * 2 - 3  # two launches a step against one per check period
+        for a, b in zip(v0, v1):
+            if precision == P.FP32_BULK:
+                assert np.array_equal(a, b)
+            else:
+                assert rel_err(a, b) <= ITER_TOL
     g.close()
