@@ -141,3 +141,22 @@ def test_step_kernel_equals_the_per_pass_kernels(name, algorithm):
             else:
                 assert rel_err(a, b) <= ITER_TOL
     g.close()
+
+
+@pytest.mark.parametrize("algorithm", ["halpern", "averaged"])
+def test_handed_off_lps_end_as_on_a_sharing_handle(algorithm):
+    """A batch hands an LP off to the single-LP path on the per-pass kernels: the bits of a handle that shares the GPU."""
+    lps = [lpgen.small_face_lp(s) for s in range(6)]
+    kw = dict(algorithm=P.HALPERN if algorithm == "halpern" else P.AVERAGED)
+    B = P.Batch(lps)
+    B.set_handoff(16, 128)
+    reps = B.solve(**kw)
+    handed = [k for k in range(len(lps)) if B.handed_off(k)]
+    assert handed
+    for k in handed:
+        g = P.lp_from_dict(lps[k])
+        g.set_gpu_sharing(True)
+        rep = g.solve(**kw)
+        assert rep["iters"] == reps[k]["iters"] and rep["pobj"] == reps[k]["pobj"] and rep["rel_kkt"] == reps[k]["rel_kkt"]
+        g.close()
+    B.close()
