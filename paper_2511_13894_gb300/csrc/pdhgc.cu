@@ -1002,15 +1002,17 @@ int fill_steps(pdhgc_lp* lp, const pdhgc_lp::Steps& sp, bool indices, cudaStream
 // without room for the entries it lost at 2.2M (FP64 31.3 -> 41.5, FP32 28.1 ->
 // 36.1): there the launches of many warps hide more latency than 16 warps a SM.
 // Flow order where no row is hot, and up to kFlowMaxNnz nonzeros with hot rows:
-// above, copying the hot entries costs more than the barriers.  Measured with
-// hot rows (power law, transportation, dense; us per iteration, median of 8
-// handles, barrier -> flow): FP64 16k 6.7 -> 5.9, 30k 6.8 -> 5.8 and 6.9 -> 6.7,
-// 32k 6.8 -> 6.9, 40k 7.0 -> 6.2; 48k 7.2 -> 7.1, 60k 7.3 -> 9.0, 64k 7.9 -> 8.6,
-// 80k 7.5 -> 9.1 and 7.2 -> 10.9, 160k 7.9 -> 8.9; FP32 40k 7.7 -> 6.3, 48k 8.8 ->
-// 9.9, 64k 9.1 -> 9.4 and (transportation) 8.0 -> 6.5, 80k 9.2 -> 9.1, 120k 6.9 ->
-// 13.0.  Between 40k and 80k the two overlap; flow gains little there and can
-// lose half.
-constexpr int64_t kFlowMaxNnz = 40960;
+// far above, copying the hot entries costs more than the barriers.  Measured
+// with hot rows (power law, transportation, dense; 8 to 10 handles each, median
+// time of flow / barrier per iteration, FP64 and FP32): 16k nonzeros 0.88 and
+// 0.97; 30k to 40k 0.85 to 1.02 and 0.82 to 1.01; 48k 0.81, 0.98 and 0.83, 1.05;
+// 60k to 66k 0.90 to 1.24 and 0.79 to 1.13 (14 LPs, mean 1.02); 80k 1.15 to 1.52
+// and 0.99 to 1.15; 90k to 120k 1.08 to 1.53 and 1.01 to 1.87; 160k 1.07, 1.13
+// and 0.98, 1.19.  The line lies where the mean crosses 1.  Around it the two do
+// not separate by size: barrier order takes the same on every handle (2000 x
+// 8000 power law 7.9 us), flow 6.5 to 9.2 with the LP and with where the handle's
+// entries lie in L2.
+constexpr int64_t kFlowMaxNnz = 65536;
 // At least this much work per CTA (nonzeros, and two for each row and column):
 // small LPs leave SMs to other handles (200 x 500: 8, 16 and 152 CTAs within 2%)
 constexpr int kStepCtaWork = 128;

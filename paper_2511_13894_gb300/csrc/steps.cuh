@@ -23,8 +23,9 @@
 //     are copied to shared memory once per CTA and pass.
 // Loop time per iteration, before (two launches) and now, us (GB300, Halpern):
 //   FP64  200 x 500 random face 7.9 -> 3.4 (flow), 5000 x 17500 with bounds
-//         (averaged) 10.3 -> 5.1 (flow), 2000 x 8000 power law 13.8 -> 7.9
-//         (barrier), 20k x 80k power law 18.7 -> 12.7 (barrier)
+//         (averaged) 10.3 -> 5.1 (flow), 2000 x 8000 power law 13.8 -> 6.5 to 9.2
+//         (flow; it depends on where the entries lie in L2), 20k x 80k power law
+//         18.7 -> 12.7 (barrier)
 //   FP32  20k x 80k power law (averaged) 17.7 -> 12.4 (barrier)
 #pragma once
 #include "kernels.cuh"
