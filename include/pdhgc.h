@@ -335,7 +335,7 @@ int pdhgc_set_gpu_sharing(pdhgc_lp* lp, int32_t shared);
  *     each pass;
  *   PDHGC_LOOP_FLOW    (2): the same without barriers, each gather waiting for
  *     the values it reads.
- * A query for measurement and tests.  Errors: INVALID_ARG.
+ * The FP32 layout of the latter two is planned by the first FP32 solve.  A query for measurement and tests.  Errors: INVALID_ARG.
  */
 #define PDHGC_LOOP_PASSES  0
 #define PDHGC_LOOP_BARRIER 1

@@ -752,6 +752,10 @@ struct pdhgc_lp {
     size_t entry_bytes = 0;  // of both, fx first
   } steps64, steps32;
   bool step_flow = false;
+  struct Segments {
+    Csr A, T;  // row pointers and segments only
+  };
+  std::unique_ptr<Segments> segs32;  // until the FP32 layout is planned (by the first FP32 solve)
   bool shared_gpu = false;  // pdhgc_set_gpu_sharing: the per-pass kernels, whatever the plans
   int step_ctas = 0;
   size_t step_smem_max = 0;
@@ -1005,8 +1009,8 @@ int fill_steps(pdhgc_lp* lp, const pdhgc_lp::Steps& sp, bool indices, cudaStream
 // far above, copying the hot entries costs more than the barriers.  Measured
 // with hot rows (power law, transportation, dense; 8 to 10 handles each, median
 // time of flow / barrier per iteration, FP64 and FP32): 16k nonzeros 0.88 and
-// 0.97; 30k to 40k 0.85 to 1.02 and 0.82 to 1.01; 48k 0.81, 0.98 and 0.83, 1.05;
-// 60k to 66k 0.90 to 1.24 and 0.79 to 1.13 (14 LPs, mean 1.02); 80k 1.15 to 1.52
+// 0.97; 30k to 40k 0.85 to 1.03 and 0.82 to 1.07; 48k 0.81, 0.98 and 0.83, 1.05;
+// 60k to 66k 0.90 to 1.24 and 0.79 to 1.13 (14 ratios, mean 1.02); 80k 1.15 to 1.52
 // and 0.99 to 1.15; 90k to 120k 1.08 to 1.53 and 1.01 to 1.87; 160k 1.07, 1.13
 // and 0.98, 1.19.  The line lies where the mean crosses 1.  Around it the two do
 // not separate by size: barrier order takes the same on every handle (2000 x
@@ -1092,6 +1096,19 @@ int setup_steps_one(pdhgc_lp* lp, pdhgc_lp::Steps& sp, const Csr& A, const Csr& 
   return PDHGC_OK;
 }
 
+// a matrix without its entries
+Csr segments_of(Csr&& C) {
+  Csr S;
+  S.rows = C.rows;
+  S.nnz = C.nnz;
+  S.cta_rows = C.cta_rows;
+  S.long_rows = C.long_rows;
+  S.nslices = C.nslices;
+  S.row_ptr = std::move(C.row_ptr);
+  S.slice_w = std::move(C.slice_w);
+  return S;
+}
+
 int setup_steps(pdhgc_lp* lp, const Csr& A, const Csr& T, cudaStream_t st) {
   int dev = 0, sms = 0, smem = 0, coop = 0;
   CK(cudaGetDevice(&dev));
@@ -1103,8 +1120,17 @@ int setup_steps(pdhgc_lp* lp, const Csr& A, const Csr& T, cudaStream_t st) {
   if (!coop || 16.0 * (double)lp->nnz > room) return PDHGC_OK;
   lp->step_ctas = (int)std::min<int64_t>(sms, std::max<int64_t>(1, (lp->nnz + 2 * ((int64_t)lp->m + lp->n)) / kStepCtaWork));
   RET(lp->alloc(&lp->step_part, 2 * (size_t)lp->step_ctas));
-  if (24.0 * (double)lp->nnz <= room) RET(setup_steps_one<double>(lp, lp->steps64, A, T, st));
-  return setup_steps_one<float>(lp, lp->steps32, A, T, st);
+  lp->segs32.reset(new pdhgc_lp::Segments());
+  return 24.0 * (double)lp->nnz <= room ? setup_steps_one<double>(lp, lp->steps64, A, T, st) : PDHGC_OK;
+}
+
+// The FP32 layout, on the first FP32 solve: most handles run in one precision,
+// and the FP64 layout serves every solve (the power iteration).  Both at
+// creation made it 0.46 -> 0.55 ms for a 200 x 500 LP
+int ensure_steps32(pdhgc_lp* lp) {
+  if (!lp->segs32) return PDHGC_OK;
+  const std::unique_ptr<pdhgc_lp::Segments> segs = std::move(lp->segs32);
+  return setup_steps_one<float>(lp, lp->steps32, segs->A, segs->T, lp->stream);
 }
 
 DevModel model_orig(const pdhgc_lp* lp) {
@@ -2333,6 +2359,10 @@ int pdhgc::lp_create(pdhgc_lp** out, int32_t m, int32_t n, int64_t nnz, const in
   CK(cudaMemsetAsync(lp->step_seq, 0, sizeof(unsigned) * (kStepBar + 1), st));
   if (own_gpu) RET(setup_steps(lp.get(), P.A, P.AT, st));
   CK(cudaStreamSynchronize(st));  // the host vectors of P go out of scope
+  if (lp->segs32) {
+    lp->segs32->A = segments_of(std::move(P.A));
+    lp->segs32->T = segments_of(std::move(P.AT));
+  }
   pdhgc_default_params(&lp->params);
   *out = lp.release();
   return PDHGC_OK;
@@ -2352,6 +2382,7 @@ int pdhgc_solve(pdhgc_lp* lp, const pdhgc_params* params, pdhgc_report* out) {
   RET(setup_scaling(lp, p));
   if (p.precision == PDHGC_FP32_BULK) {
     RET(ensure_fp32(lp));
+    RET(ensure_steps32(lp));
     RET(convert_fp32(lp, lp->stream));
   }
   PhaseInit pi{};
@@ -2626,6 +2657,7 @@ int pdhgc_set_state(pdhgc_lp* lp, const void* buf, size_t bytes) {
   RET(setup_scaling(lp, h.params));
   if (h.params.precision == PDHGC_FP32_BULK) {
     RET(ensure_fp32(lp));
+    RET(ensure_steps32(lp));
     RET(convert_fp32(lp, st));
   }
   RET(take_error(lp));

@@ -160,3 +160,23 @@ def test_handed_off_lps_end_as_on_a_sharing_handle(algorithm):
         assert rep["iters"] == reps[k]["iters"] and rep["pobj"] == reps[k]["pobj"] and rep["rel_kkt"] == reps[k]["rel_kkt"]
         g.close()
     B.close()
+
+
+def test_a_handle_lays_out_the_precision_it_runs_in():
+    """Creation launches the two fills of the FP64 step layout and the SELL fills; the FP32 layout's two come with the
+    first FP32 solve, whose bits those of later ones are."""
+    lp = lpgen.small_face_lp(2)
+    g = P.lp_from_dict(lp)
+    assert g.kernel_launches() == 2 * 2 + 2
+    assert g.get_loop_kernel(P.FP64) == P.LOOP_FLOW and g.get_loop_kernel(P.FP32_BULK) == P.LOOP_PASSES
+    kw = dict(max_iters=70, eps_rel=-1.0, algorithm=P.HALPERN)
+    counts, xs = [], []
+    for precision in (P.FP64, P.FP64, P.FP32_BULK, P.FP32_BULK):
+        before = g.kernel_launches()
+        g.solve(precision=precision, **kw)
+        counts.append(g.kernel_launches() - before)
+        xs.append(g.get_iterates()["x"])
+    assert counts[0] == counts[1] and counts[2] == counts[3] + 2
+    assert np.array_equal(xs[0], xs[1]) and np.array_equal(xs[2], xs[3])
+    assert g.get_loop_kernel(P.FP32_BULK) == P.LOOP_FLOW
+    g.close()
