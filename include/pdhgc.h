@@ -365,8 +365,12 @@ int pdhgc_set_wait_limit(pdhgc_lp* lp, int64_t polls);
  * `cuda_stream`, which the call synchronises.  The inputs are not
  * validated beyond NULL and size checks (use pdhgc_lp_create for that).
  * Scratch (n + 15 * 608 + 16 doubles) is taken with cudaMallocAsync on
- * the stream and freed on it before returning.  A'y is accumulated with
- * atomic adds, so results may differ from run to run in the last bits.
+ * the stream and freed on it before returning.  The call does not wait for
+ * that free: the device's default memory pool keeps the scratch mapped, for
+ * the next call or any other allocation from the pool, until the caller next
+ * synchronises (which then takes about 90 us longer) or trims the pool.
+ * A'y is accumulated with atomic adds, so results may differ from run to run
+ * in the last bits.
  * Errors: INVALID_ARG, OOM, CUDA.
  */
 int pdhgc_kkt_eval(int32_t m, int32_t n, int64_t nnz, const int64_t* row_ptr, const int32_t* col_idx,
@@ -385,7 +389,7 @@ int pdhgc_kkt_eval(int32_t m, int32_t n, int64_t nnz, const int64_t* row_ptr, co
  * TOO_LARGE (below), CUDA; never OOM.  Further:
  *  - n must be <= 262,144 (1 << 18); a larger n returns PDHGC_ERR_TOO_LARGE
  *    without touching the device.
- *  - The scratch is a file-scope device array of 2,203,776 bytes ((1 << 18)
+ *  - The scratch is a file-scope device array of 2,170,240 bytes ((1 << 18)
  *    + 15 * 608 + 16 doubles) that every GPU which loads the library holds
  *    until the process exits.  The call itself allocates nothing and calls
  *    no cudaMalloc, cudaFree or allocating library routine.

@@ -275,9 +275,13 @@ extern "C" int pdhgc_kkt_eval(int32_t m, int32_t n, int64_t nnz, const int64_t* 
     return pdhgc::set_error_detail(PDHGC_ERR_OOM, std::string("cudaMallocAsync: ") + cudaGetErrorString(e));
   pdhgc::EvalInput in{m, n, nnz, row_ptr, col_idx, val, b, c, lb, ub, sense, x, y};
   rc = pdhgc::kkt_eval_run(in, static_cast<double*>(scratch), st, out, detail);
-  // the evaluation has ended (its results were read): no synchronisation behind
-  // the free, at which the device's default pool would unmap the scratch and
-  // the next call map it again, 165 us of an evaluation of the 100k x 400k LP
+  // The evaluation has ended (its results were read): no synchronisation behind
+  // the free, at which the device's default pool would unmap the scratch for the
+  // next call to map it again.  100k x 400k LP, us a call, new inputs each time:
+  // 123 one after another, 230 where the caller synchronises before each, 320
+  // with the caller's synchronisation behind it counted in; with a
+  // synchronisation here 300 in every case; 990 to 1,010 before the kernels of
+  // this file.  Inputs out of L2 add 10
   cudaFreeAsync(scratch, st);
   if (rc != PDHGC_OK) return pdhgc::set_error_detail(rc, detail);
   return PDHGC_OK;
