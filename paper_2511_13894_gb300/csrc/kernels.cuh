@@ -458,27 +458,30 @@ using SpmvMat = SpmvMatT<double>;
 constexpr int kBatch = PDHGC_GATHER_BATCH;
 
 // acc += sum over k = k0, k0+step, ... < k1 of val[k] * gathered(col[k]), in
-// that order, with kBatch gathers in flight per lane (CSR rows)
+// that order, with kBatch gathers in flight per lane (CSR rows).  The
+// distance to k1 is what is compared: an index up to two batches past the row's
+// end can pass 2^31
 template <class Op>
 __device__ __forceinline__ void row_dot_global(const Op& op, typename Op::Acc& acc, double rc,
                                                const typename Op::VT* __restrict__ val,
-                                               const int* __restrict__ col, int k0, int k1, int step) {
+                                               const int* __restrict__ col, unsigned k0, unsigned k1, int step) {
   constexpr int NG = Op::NG;
   using VT = typename Op::VT;
   using GT = typename Op::GT;
   // the next batch's matrix entries are requested while this batch's gathers
   // are in flight: a long row is a chain of batches on one warp
+  int left = (int)(k1 - k0);
   VT v[kBatch];
   int c[kBatch];
 #pragma unroll
   for (int u = 0; u < kBatch; ++u) {
     c[u] = -1;
-    if (k0 + u * step < k1) {
+    if (u * step < left) {
       v[u] = ld_stream(val + k0 + u * step);
       c[u] = ld_stream(col + k0 + u * step);
     }
   }
-  for (int k = k0; k < k1; k += kBatch * step) {
+  for (unsigned k = k0; left > 0; k += kBatch * step, left -= kBatch * step) {
     GV<GT, NG> g[kBatch];
 #pragma unroll
     for (int u = 0; u < kBatch; ++u)
@@ -490,7 +493,7 @@ __device__ __forceinline__ void row_dot_global(const Op& op, typename Op::Acc& a
 #pragma unroll
     for (int u = 0; u < kBatch; ++u) {
       cn[u] = -1;
-      if (k + (kBatch + u) * step < k1) {
+      if ((kBatch + u) * step < left) {
         vn[u] = ld_stream(val + k + (kBatch + u) * step);
         cn[u] = ld_stream(col + k + (kBatch + u) * step);
       }
