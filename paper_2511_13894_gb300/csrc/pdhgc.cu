@@ -2381,8 +2381,8 @@ int pdhgc_solve(pdhgc_lp* lp, const pdhgc_params* params, pdhgc_report* out) {
   lp->have_dual = false;
   RET(setup_scaling(lp, p));
   if (p.precision == PDHGC_FP32_BULK) {
-    RET(ensure_fp32(lp));
     RET(ensure_steps32(lp));
+    RET(ensure_fp32(lp));
     RET(convert_fp32(lp, lp->stream));
   }
   PhaseInit pi{};
@@ -2656,8 +2656,8 @@ int pdhgc_set_state(pdhgc_lp* lp, const void* buf, size_t bytes) {
   // must reproduce the saved factors bit for bit
   RET(setup_scaling(lp, h.params));
   if (h.params.precision == PDHGC_FP32_BULK) {
-    RET(ensure_fp32(lp));
     RET(ensure_steps32(lp));
+    RET(ensure_fp32(lp));
     RET(convert_fp32(lp, st));
   }
   RET(take_error(lp));
