@@ -250,8 +250,8 @@ __global__ void __launch_bounds__(kGThreads) k_guide_forward(const GuideBf16* __
 
 // ---------------------------------------------------------------------------
 // Inference on the 5th-generation tensor cores: tcgen05.mma with operands in
-// shared memory and FP32 accumulators in tensor memory.  One CTA per SM
-// (persistent over 128-row tiles), 4 warps; thread t owns row t of a tile.
+// shared memory and FP32 accumulators in tensor memory.  Up to four CTAs per SM
+// (persistent over 128-row tiles), 4 warps each; thread t owns row t of a tile.
 // Layer 1: D1[128 x 64] = X[128 x 32] W1'; layer 2: D2[128 x 64] = A1[128 x 64]
 // W2'.  Operands use the K-major layout without swizzle: core matrices of
 // 8 rows x 16 bytes (8 BF16) stored contiguously, the K-adjacent cores 128
@@ -867,7 +867,7 @@ __device__ __forceinline__ void train_barrier(unsigned* bar, unsigned target, in
 // take the gradient, the others (none with kAll) only fold: they are a variant
 // of their own since the test for them costs the large batches 1.2 us a step
 // (4096 rows: 10.5 and 11.7).  Two launches per step took 22.5 us (80k rows,
-// batches of 4096), most of it latency; here a step takes 11.6: the next step's
+// batches of 4096), most of it latency; here a step takes 11.3: the next step's
 // samples are read while the barrier is waited for.  coef: (c1, c2) of each
 // step; bar: 0 at launch.
 template <bool kAll>
